@@ -1,0 +1,299 @@
+// The cell test of the bucket path for models without atomics and without warp
+// or grid barriers: every bucket's cells are decided in shared memory, without
+// sorting the bucket's keys.
+//
+// A cell is racy iff it has a write and either two blocks meet in it or, inside
+// one block, some barrier interval holds two threads and a write (the
+// cell-level form of the pair rule in include/rc.h).  Every cell of a bucket has
+// its own slot of a table in shared memory (the slot is the rest of the cell
+// hash below the bucket bits, so equal slots are equal cells), and a key's low
+// word holds its interval, block, thread and kind:
+//   1. every write stores its low word in its cell's slot; whichever store wins
+//      is the cell's representative write;
+//   2. every key compares itself with the representative.  Another block, or
+//      another thread in the representative's interval: the cell is racy.
+//      Another thread in another interval: the cell has two threads.  A write in
+//      another interval: the cell has writes in two intervals.
+//      A cell that is not racy by now races only if both marks are there (with
+//      one write interval the representative stands for it, and every key was
+//      compared with it): few cells in practice;
+//   3. these candidate cells are numbered, and 1 and 2 are done again per
+//      (candidate cell, barrier interval): a key that finds another thread's
+//      write in its own interval makes the cell racy.
+// A representative decides exactly: if an interval (or cell) has a write and two
+// threads (or blocks), at least one of its keys differs from whichever write
+// was kept.  Which store wins does not matter, so the stores need no order.
+//
+// What bounds it: one read of every key (8 bytes); about 78 warp instructions per
+// 32 keys keep the issue slots 76 % busy.  On the 4096 x 256 random affine model
+// (578 M keys, 2^17 buckets of 4,400 keys) 1.35 ms, where the counting sort of
+// every bucket and the cell scan that it replaces there took 3.52 + 1.66 ms; on
+// 49 M keys with hot cells 0.26 ms against 1.63 + 0.22 ms.  Blocks of 256 threads
+// with 20 keys each in registers, 4 per SM, were the fastest split without spills
+// (512 threads, 2 per SM: 1.95 ms; 384 threads with 16 keys, 3 per SM: 1.51 ms):
+// the barriers between the steps stall fewer warps.
+#include <cuda_runtime.h>
+
+#include "fold.cuh"
+#include "kernels.h"
+
+namespace rc {
+
+namespace {
+
+constexpr unsigned FULL = 0xffffffffu;
+constexpr int kFltThreads = 256;
+constexpr int kFltBlocks = 4;                      // blocks per SM
+constexpr int kFltKPT = 20;                        // keys per thread held in registers
+constexpr int kFltStreamKPT = 12;                  // keys per thread and step of a larger bucket
+constexpr unsigned kFltCap = kFltThreads * kFltKPT;
+static_assert((1 << kFilterMaxSlotBits) / 32 <= kFltThreads, "a word of a bit mask per thread");
+
+// inverse of the odd hash multiplier modulo 2^64 (Newton's iteration: each step
+// doubles the number of correct low bits)
+constexpr uint64_t hash_inverse() {
+  uint64_t x = kCellHashMul;   // correct to 3 bits
+  for (int i = 0; i < 5; ++i) x *= 2ull - kCellHashMul * x;
+  return x;
+}
+static_assert(hash_inverse() * kCellHashMul == 1ull, "inverse of the cell hash multiplier");
+
+// words of the representative table: a slot per cell, and room for at least
+// 256 candidate cells of 16 intervals each
+__host__ __device__ __forceinline__ unsigned table_words(uint32_t r) {
+  return r < 12 ? 4096u : (1u << r);
+}
+__host__ __device__ __forceinline__ unsigned mask_words(uint32_t r) { return r < 5 ? 1u : (1u << (r - 5)); }
+// (four words behind the table: the slot of padding keys)
+size_t filter_smem(uint32_t r) { return ((size_t)table_words(r) + 4 + 5 * (size_t)mask_words(r) + 1) * sizeof(unsigned); }
+
+// One block per bucket.  A bucket of at most kFltCap keys is held in registers
+// as (low word, slot); a larger one is read again in every step.  Key slots of
+// a thread past the bucket's end repeat its first key (the same instance, which
+// changes nothing), so no step tests for them; PAD: the bucket holds padding
+// keys (the unpartitioned single bucket), held as reads of the word behind the table.
+template <bool PAD, bool REGS>
+__device__ __forceinline__ void filter_bucket(const FilterArgs& a, const uint64_t* src, uint64_t len) {
+  extern __shared__ __align__(16) unsigned s_tab[];
+  const unsigned tw = table_words(a.r), mw = mask_words(a.r);
+  unsigned* s_two = s_tab + tw + 4;     // cells with two threads of a block, a bit per slot
+  unsigned* s_wi = s_two + mw;          // cells with writes in two intervals, then the candidate cells
+  unsigned* s_racy = s_wi + mw;         // racy cells
+  unsigned* s_hot = s_racy + mw;        // racy candidate cells, a bit per candidate
+  unsigned* s_rank = s_hot + mw + 1;    // candidate cells before each word of s_wi
+  __shared__ unsigned s_wsum[kFltThreads / 32];
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  const uint32_t pb = a.s.phase_bits, bb = a.s.block_bits, tb = a.s.thread_bits;
+  // a low word's fields: (block, thread), block, interval
+  const unsigned m_bt = (unsigned)(((1ull << (bb + tb)) - 1ull) << 1),
+                 m_b = (unsigned)(((1ull << bb) - 1ull) << (1 + tb)),
+                 m_p = (unsigned)(((1ull << pb) - 1ull) << (1 + tb + bb));
+  const uint32_t cs = a.s.cell_shift;
+  const unsigned smask = (1u << a.r) - 1u;
+  const unsigned lmask = cs < 32 ? (1u << cs) - 1u : ~0u;
+  // low word and slot of a key (the low r bits of the hash depend on the low bits
+  // of the cell alone)
+  auto unpack = [&](uint64_t k, unsigned& kl, unsigned& sl) {
+    kl = (uint32_t)k & lmask;
+    sl = (__funnelshift_rc((uint32_t)k, (uint32_t)(k >> 32), cs) * (uint32_t)kCellHashMul) & smask;
+    if (PAD && k == kSentinel) {
+      sl = tw;
+      kl = 0;
+    }
+  };
+  unsigned rl[kFltKPT], rs[kFltKPT];   // (REGS) the bucket
+  const int nq = REGS ? (int)((len + kFltThreads - 1) / kFltThreads) : 0;
+  if constexpr (REGS) {
+    const uint64_t* p = src + tid;
+    uint64_t k[kFltKPT];
+    const uint64_t k0 = __ldg(src);
+#pragma unroll
+    for (int q = 0; q < kFltKPT; ++q) {
+      if (q >= nq) break;
+      k[q] = k0;
+      if (q < nq - 1 || (unsigned)(q * kFltThreads + tid) < (unsigned)len) k[q] = __ldg(p + q * kFltThreads);
+    }
+#pragma unroll
+    for (int q = 0; q < kFltKPT; ++q) {
+      if (q >= nq) break;
+      unpack(k[q], rl[q], rs[q]);
+    }
+  }
+  // f(low word, slot) for the keys of the bucket
+  auto each = [&](auto&& f) {
+    if constexpr (REGS) {
+#pragma unroll
+      for (int q = 0; q < kFltKPT; ++q) {
+        if (q >= nq) break;
+        // (opaque to the compiler, which would keep what it derives from the pair in
+        // one step for the next one and run out of registers)
+        asm volatile("" : "+r"(rl[q]), "+r"(rs[q]));
+        f(rl[q], rs[q]);
+      }
+    } else {
+      const uint64_t k0 = __ldg(src);
+      for (uint64_t i = tid; i < len; i += kFltStreamKPT * kFltThreads) {
+        uint64_t k[kFltStreamKPT];
+#pragma unroll
+        for (int u = 0; u < kFltStreamKPT; ++u)
+          k[u] = i + u * kFltThreads < len ? __ldg(src + i + u * kFltThreads) : k0;
+#pragma unroll
+        for (int u = 0; u < kFltStreamKPT; ++u) {
+          unsigned kl, sl;
+          unpack(k[u], kl, sl);
+          f(kl, sl);
+        }
+      }
+    }
+  };
+  auto clear_table = [&](unsigned words) {
+    for (unsigned i = 4 * tid; i < words; i += 4 * kFltThreads)
+      *reinterpret_cast<uint4*>(s_tab + i) = make_uint4(0, 0, 0, 0);
+  };
+  auto mark = [&](unsigned* bits, unsigned i) {
+    const unsigned bit = 1u << (i & 31u);
+    if (!(bits[i >> 5] & bit)) atomicOr(&bits[i >> 5], bit);
+  };
+  // (the slots rounded up to whole 16-byte stores lie inside the table)
+  clear_table(PAD ? tw + 4u : ((1u << a.r) + 3u) & ~3u);
+  for (unsigned i = tid; i < 4 * mw + 1; i += kFltThreads) s_two[i] = 0;
+  __syncthreads();
+  // 1. the representative write of every written cell (a write's low word is odd)
+  bool any = false;
+  each([&](unsigned k, unsigned s) {
+    if (k & 1u) {
+      s_tab[s] = k;
+      any = true;
+    }
+  });
+  if (!__syncthreads_or(any)) return;   // no write: nothing can race
+  // 2. every key against its cell's representative
+  any = false;
+  each([&](unsigned k, unsigned s) {
+    const unsigned rep = s_tab[s];
+    const unsigned d = rep ^ k;
+    if (rep != 0u && (d & ((k & 1u) ? m_bt | m_p : m_bt)) != 0u) {
+      any = true;
+      if (d & m_bt) mark((d & m_b) || !(d & m_p) ? s_racy : s_two, s);
+      if ((k & 1u) && (d & m_p)) mark(s_wi, s);
+    }
+  });
+  if (!__syncthreads_or(any)) return;   // every written cell has one thread and interval
+  // 3. the candidate cells numbered in slot order; at most one word of a bit
+  // mask per thread
+  unsigned cand = 0;
+  if (tid < (int)mw) {
+    cand = s_two[tid] & s_wi[tid] & ~s_racy[tid];
+    s_wi[tid] = cand;
+  }
+  if (__syncthreads_or(cand != 0u)) {
+    const unsigned c = __popc(cand);
+    unsigned x = c;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const unsigned y = __shfl_up_sync(FULL, x, o);
+      if (lane >= o) x += y;
+    }
+    if (lane == 31) s_wsum[w] = x;
+    __syncthreads();
+    unsigned before = 0, ncand = 0;
+#pragma unroll 4
+    for (int i = 0; i < kFltThreads / 32; ++i) {
+      if (i < w) before += s_wsum[i];
+      ncand += s_wsum[i];
+    }
+    if (tid < (int)mw) s_rank[tid] = before + x - c;
+    __syncthreads();
+    // the entry (candidate << pb | interval) of a key, ~0 if its cell is no candidate
+    auto entry = [&](unsigned k, unsigned s) -> unsigned {
+      if (PAD && s == tw) return ~0u;
+      const unsigned m = s_wi[s >> 5];
+      if (!((m >> (s & 31u)) & 1u)) return ~0u;
+      return ((s_rank[s >> 5] + __popc(m & ((1u << (s & 31u)) - 1u))) << pb) | (unsigned)((uint64_t)k >> (1 + bb + tb));
+    };
+    // windows of tw entries of the table
+    for (unsigned e0 = 0; e0 < (ncand << pb); e0 += tw) {
+      const unsigned used = min(tw, (ncand << pb) - e0);
+      clear_table((used + 3u) & ~3u);
+      __syncthreads();
+      each([&](unsigned k, unsigned s) {
+        if (k & 1u) {
+          const unsigned e = entry(k, s) - e0;
+          if (e < used) s_tab[e] = k;
+        }
+      });
+      __syncthreads();
+      each([&](unsigned k, unsigned s) {
+        const unsigned e = entry(k, s) - e0;
+        if (e < used) {
+          const unsigned rep = s_tab[e];
+          if (rep != 0u && ((rep ^ k) & m_bt) != 0u) mark(s_hot, (e + e0) >> pb);
+        }
+      });
+      __syncthreads();
+    }
+  }
+  // the racy cells: counted, and the smallest by value kept.  Slot s of bucket b
+  // has hash (part | b | s), whose cell is hash * inverse mod 2^(cell bits).
+  const uint64_t inv = hash_inverse();
+  unsigned count = 0;
+  unsigned long long first = ~0ull;
+  if (tid < (int)mw) {
+    unsigned m = s_racy[tid];
+    if (cand) {
+      // the racing candidates of this word back to their slots
+      const unsigned r0 = s_rank[tid];
+      unsigned hot = __funnelshift_r(s_hot[r0 >> 5], s_hot[(r0 >> 5) + 1], r0 & 31u);
+      for (unsigned c = cand; c && hot; c &= c - 1u, hot >>= 1)
+        if (hot & 1u) m |= c & (0u - c);
+    }
+    count = __popc(m);
+    while (m) {
+      const unsigned slot = 32u * tid + (unsigned)__ffs(m) - 1u;
+      m &= m - 1u;
+      const uint64_t h = a.part_hash | ((uint64_t)blockIdx.x << a.r) | slot;
+      const uint64_t cell = (h * inv) & a.hmask;
+      if (a.s.n_models) {
+        DevResult* r = result_of(a.s, cell);
+        atomicAdd(&r->racy_cells, 1ull);
+        atomicMin(&r->hash_cell, (unsigned long long)cell);
+      } else {
+        first = min(first, (unsigned long long)cell);
+      }
+    }
+  }
+  if (a.s.n_models) return;
+  count = __reduce_add_sync(FULL, count);
+  if (count == 0) return;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) first = min(first, __shfl_xor_sync(FULL, first, o));
+  if (lane == 0) {
+    atomicAdd(&a.s.res->racy_cells, (unsigned long long)count);
+    atomicMin(&a.s.res->hash_cell, first);
+  }
+}
+
+template <bool PAD>
+__global__ void __launch_bounds__(kFltThreads, kFltBlocks) bucket_filter_kernel(FilterArgs a) {
+  const uint64_t lo = a.boff[blockIdx.x], hi = a.boff[blockIdx.x + 1];
+  if (hi < lo + 2) return;              // a race needs two keys
+  if (hi - lo <= (uint64_t)kFltCap) filter_bucket<PAD, true>(a, a.keys_in + lo, hi - lo);
+  else filter_bucket<PAD, false>(a, a.keys_in + lo, hi - lo);
+}
+
+}  // namespace
+
+cudaError_t launch_bucket_filter(const FilterArgs& a, uint32_t D, cudaStream_t st) {
+  if (a.r > kFilterMaxSlotBits || a.s.cell_shift > kFilterMaxLowBits) return cudaErrorInvalidValue;
+  // an unpartitioned bucket holds padding keys, which take the table's last word
+  const bool pad = D == 0;
+  const void* fn = pad ? reinterpret_cast<const void*>(bucket_filter_kernel<true>)
+                       : reinterpret_cast<const void*>(bucket_filter_kernel<false>);
+  const cudaError_t e = ensure_kernel_smem(fn, filter_smem(kFilterMaxSlotBits));
+  if (e != cudaSuccess) return e;
+  if (pad) bucket_filter_kernel<true><<<1, kFltThreads, filter_smem(a.r), st>>>(a);
+  else bucket_filter_kernel<false><<<1u << D, kFltThreads, filter_smem(a.r), st>>>(a);
+  return cudaGetLastError();
+}
+
+}  // namespace rc

@@ -345,8 +345,20 @@ constexpr uint64_t kBucketTarget = kFoldCap / 2 + kFoldCap / 16;   // planned me
 constexpr int kBucketHistTile = 16384;              // keys per block of the pass-B histogram
 constexpr int kPartTileHost = kSortThreadsHost * 16;    // keys per tile of the partition passes
 
+// The cell test in shared memory (filter.cu).  The target keeps a bucket's keys
+// inside its block's registers (5,120) with room for the spread; 6,000 and 9,000
+// keys with larger blocks measured slower.  Fewer keys per bucket than
+// kFilterMinKeys would clear and scan a mostly empty table: the local sort's
+// buckets then cost less.
+constexpr uint32_t kFilterMaxSlotBits = 13;         // table slots of a bucket: 32 KB of 4-byte words
+constexpr uint32_t kFilterMaxLowBits = 32;          // (interval, block, thread, kind) bits: a table word
+constexpr uint64_t kFilterTarget = 4700;            // planned mean keys per bucket (at most)
+constexpr uint64_t kFilterMinKeys = 512;            // ... and at least, where the cell bits ask for more buckets
+constexpr uint64_t kFilterOnePassKeys = 48 * 1024;  // ... and at most, where one partition pass does
+
 struct BucketPlan {
   bool on = false;
+  bool filter = false;            // the cells are decided by the table test instead of local sort and scan
   uint32_t cb = 0, dA = 0, dB = 0, D = 0, r = 0, rbin = 0;
   uint64_t n = 0;                 // key slots (padding included)
   uint64_t tiles_b = 0, tiles_h = 0;   // grid bounds of pass B and its histogram
@@ -360,7 +372,9 @@ struct BucketPlan {
 // host (runtime.cu): whether the bucket path applies to n keys of cb cell bits
 // (at most 2^kBucketMaxBits buckets of about kBucketTarget keys), its digit
 // widths, and its workspace section laid out from byte offset `off`
-bool plan_buckets(uint64_t n, uint64_t n_expect, uint32_t cb, size_t off, BucketPlan* bp);
+// filter_ok: the model admits the table test (no atomics, no warp or grid
+// barriers, at most kFilterMaxLowBits key bits below the cell)
+bool plan_buckets(uint64_t n, uint64_t n_expect, uint32_t cb, bool filter_ok, size_t off, BucketPlan* bp);
 
 
 struct WorkspacePlan {

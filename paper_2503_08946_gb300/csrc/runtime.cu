@@ -223,15 +223,41 @@ bool bucket_path_allowed(uint32_t phase_bits, const rc_check_opts* opts) {
   return true;
 }
 
+// whether a model (or a batch pack) admits the cell test in shared memory
+static bool filter_allowed(bool atomics_or_scopes, uint32_t cell_shift) {
+  return !atomics_or_scopes && cell_shift <= kFilterMaxLowBits;
+}
+
 // n key slots, of which about n_expect are kept (a hash-partitioned check keeps
 // its share): the bucket count is chosen for n_expect, the tile bounds for n
-bool plan_buckets(uint64_t n, uint64_t n_expect, uint32_t cb, size_t off, BucketPlan* bp) {
+// Bucket bits of the table test, or ~0 where it does not pay: enough buckets
+// that every cell has its own slot and a bucket's keys fit the registers.
+static uint32_t filter_bucket_bits(uint64_t n_expect, uint32_t cb) {
+  uint32_t D = 0;
+  while (D < cb && D < kBucketMaxBits && (n_expect >> D) > kFilterTarget) ++D;
+  const uint32_t need = cb > kFilterMaxSlotBits ? cb - kFilterMaxSlotBits : 0u;
+  if (need > kBucketMaxBits) return ~0u;
+  // one partition pass where its buckets stay small enough to be read again from L2
+  const uint32_t one = kBucketMaxDigitBits;
+  if (D > one && cb <= one + kFilterMaxSlotBits && (n_expect >> one) <= kFilterOnePassKeys) return one;
+  if (need > D) {
+    if ((n_expect >> need) < kFilterMinKeys) return ~0u;   // a sparse cell space: mostly empty tables
+    D = need;
+  }
+  return D;
+}
+
+bool plan_buckets(uint64_t n, uint64_t n_expect, uint32_t cb, bool filter_ok, size_t off, BucketPlan* bp) {
   *bp = BucketPlan();
   if (n == 0 || n >= (1ull << 32) || cb == 0 || cb > 62) return false;
   if (n_expect == 0 || n_expect > n) n_expect = n;
-  uint32_t D = 0;
-  while (D < cb && D < kBucketMaxBits && (n_expect >> D) > kBucketTarget) ++D;
-  if (D == kBucketMaxBits && D < cb && (n_expect >> D) > kBucketTarget) return false;   // more keys than the buckets hold
+  uint32_t D = filter_ok ? filter_bucket_bits(n_expect, cb) : ~0u;
+  bp->filter = D != ~0u;
+  if (!bp->filter) {
+    D = 0;
+    while (D < cb && D < kBucketMaxBits && (n_expect >> D) > kBucketTarget) ++D;
+    if (D == kBucketMaxBits && D < cb && (n_expect >> D) > kBucketTarget) return false;   // more keys than the buckets hold
+  }
   bp->on = true;
   bp->n = n;
   bp->cb = cb;
@@ -293,7 +319,9 @@ void plan_workspace_keys(const Model& m, const rc_check_opts* opts, uint64_t n, 
   const uint32_t part_bits = part ? bit_length(opts->part_count - 1) : 0u;
   const uint64_t n_expect = part ? n / opts->part_count + n / (16ull * opts->part_count) + 1 : n;
   if (allow_bucket && bucket_path_allowed(m.host.phase_bits, opts) && cell_bits > part_bits &&
-      plan_buckets(n, n_expect, cell_bits - part_bits, off, &p->bucket)) {
+      plan_buckets(n, n_expect, cell_bits - part_bits,
+                   filter_allowed(m.has_atomic || m.sync_scopes, m.host.cell_shift), off,
+                   &p->bucket)) {
     // the bucket path: its own section instead of the radix-sort sections
     p->zero_lo = p->bucket.zero_lo;
     p->zero_hi = p->bucket.zero_hi;
@@ -425,7 +453,8 @@ rc_status enqueue_sort(const rc::WorkspacePlan& p, uint8_t* ws, uint64_t* buf0, 
 // pass-A histogram (i_hist), around each pass, around the pass-B histogram.
 rc_status enqueue_bucketed(const rc::WorkspacePlan& p, uint8_t* ws, uint64_t* buf0, uint64_t* buf1,
                            const rc::ScanArgs& sa, cudaStream_t st, const uint64_t** final_keys,
-                           rc_ticket_s* timed = nullptr, bool hist_a_done = false) {
+                           rc_ticket_s* timed = nullptr, bool hist_a_done = false, uint32_t cell_bits = 0,
+                           uint32_t part_index = 0) {
   const rc::BucketPlan& bp = p.bucket;
   StageTimer* tm = timed ? &timed->timer : nullptr;
   auto u64 = [&](size_t off) { return reinterpret_cast<unsigned long long*>(ws + off); };
@@ -481,6 +510,34 @@ rc_status enqueue_bucketed(const rc::WorkspacePlan& p, uint8_t* ws, uint64_t* bu
     }
   }
   if (s != RC_OK) return s;
+  rc::FinishArgs fa;
+  fa.res = sa.res;
+  fa.n_models = sa.n_models;
+  fa.boff = a.boff;
+  fa.cmask = a.cmask;
+  fa.cb = bp.cb;
+  fa.D = bp.D;
+  if (bp.filter) {
+    // the cells decided bucket by bucket in shared memory; the witness reads the
+    // smallest racy cell's bucket as the partition passes left it
+    rc::FilterArgs f;
+    f.s = sa;
+    f.keys_in = fin;
+    f.boff = a.boff;
+    f.r = bp.r;
+    f.hmask = (1ull << cell_bits) - 1ull;
+    f.part_hash = cell_bits > bp.cb ? (uint64_t)part_index << bp.cb : 0ull;
+    s = cuda_status(rc::launch_bucket_filter(f, bp.D, st));
+    if (tm) { timed->i_pass_from[n_pass] = tm->n - 1; timed->i_pass_to[n_pass] = tm->n; tm->mark(); }
+    ++n_pass;
+    if (s == RC_OK) s = cuda_status(rc::launch_bucket_finish(fa, st));
+    if (timed) {
+      timed->n_pass = n_pass;
+      timed->bucketed = true;
+    }
+    *final_keys = fin;
+    return s;
+  }
   // the local sort into the other buffer, then the ordered cell scan with the
   // first racy cell kept by value, then its bucket for the witness
   rc::LocalSortArgs ls;
@@ -505,13 +562,6 @@ rc_status enqueue_bucketed(const rc::WorkspacePlan& p, uint8_t* ws, uint64_t* bu
   sc.by_cell = 1;
   sc.phase_table = 1;
   if (s == RC_OK) s = cuda_status(rc::launch_scan(sc, st));
-  rc::FinishArgs fa;
-  fa.res = sa.res;
-  fa.n_models = sa.n_models;
-  fa.boff = a.boff;
-  fa.cmask = a.cmask;
-  fa.cb = bp.cb;
-  fa.D = bp.D;
   if (s == RC_OK) s = cuda_status(rc::launch_bucket_finish(fa, st));
   if (timed) {
     timed->n_pass = n_pass;
@@ -629,7 +679,8 @@ rc_status enqueue_check(rc_model* model, const rc_check_opts* opts, uint8_t* ws,
     const uint64_t* fin = nullptr;
     rc::ScanArgs sa = scan_args(m, p, ws, 0);
     s = enqueue_bucketed(p, ws, reinterpret_cast<uint64_t*>(ws + p.keys_off[0]),
-                         reinterpret_cast<uint64_t*>(ws + p.keys_off[1]), sa, st, &fin, timed, fuse_hist);
+                         reinterpret_cast<uint64_t*>(ws + p.keys_off[1]), sa, st, &fin, timed, fuse_hist, m.host.cell_bits,
+                         opts ? opts->part_index : 0u);
     if (s != RC_OK) return s;
     if (tm) { timed->i_scan = tm->n; tm->mark(); }
     sa.keys = fin;
@@ -1141,7 +1192,9 @@ rc_status plan_batch(rc_model* const* models, size_t n, const rc_check_opts* opt
     o = align256(o + k.n_keys * 8);
     p.keys_off[1] = o;
     o = align256(o + k.n_keys * 8);
-    if (rc::bucket_path_allowed(k.pb, opts) && rc::plan_buckets(k.n_keys, k.n_keys, k.cell_bits, o, &p.bucket)) {
+    if (rc::bucket_path_allowed(k.pb, opts) && rc::plan_buckets(k.n_keys, k.n_keys, k.cell_bits,
+                                                               rc::filter_allowed(k.kb != 1 || k.sy, ps + k.pb), o,
+                                                               &p.bucket)) {
       p.zero_lo = p.bucket.zero_lo;
       p.zero_hi = p.bucket.zero_hi;
       o = p.bucket.end;
@@ -1296,7 +1349,7 @@ rc_status enqueue_batch_device(const BatchLayout& L, size_t n, const rc_check_op
     if (p.bucket.on) {
       const uint64_t* fin = nullptr;
       s = enqueue_bucketed(p, ws, reinterpret_cast<uint64_t*>(ws + p.keys_off[0]),
-                           reinterpret_cast<uint64_t*>(ws + p.keys_off[1]), sa, st, &fin);
+                           reinterpret_cast<uint64_t*>(ws + p.keys_off[1]), sa, st, &fin, nullptr, false, k.cell_bits);
       sa.keys = fin;
     } else {
       s = cuda_status(rc::launch_scan(sa, st));

@@ -1,0 +1,97 @@
+"""The cell test in shared memory (bucket path without a sort): models without
+atomics and scopes against the oracle at the edges of its buckets -- one key, the
+unpartitioned bucket, one and two partition passes, buckets above the register
+capacity (hot cells), candidate cells in several windows of the table, sixteen
+intervals, and the largest key word below the cell."""
+import pytest
+
+import oracle
+import workloads as w
+from workloads.spec import Access, Array, GLOBAL, Loop, Model, R, SHARED, Stmt, W, bid, const, it, tid
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def rc():
+    import torch
+    import paper_2503_08946_gb300 as m
+    assert torch.cuda.is_available()
+    return m
+
+
+def check(rc, model, opts=None):
+    got, exp = rc.check(model, opts), oracle.check(model)
+    assert (got.status, got.instances) == (exp.status, exp.instances) == (0, exp.instances), (model.name, got, exp)
+    assert (got.verdict, got.racy_cells, got.witness) == (exp.verdict, exp.racy_cells, exp.witness), (model.name, got, exp)
+
+
+def shared_mix(blocks, threads, cells, phases, scope=SHARED, hot=1):
+    """Cells written by one thread in several intervals and read by another one in
+    intervals with and without a write: the candidates of the test's third step,
+    about a third of them racy."""
+    a = Array("a", scope, (cells,))
+    own, other = tid.x % cells, (tid.x * 7 + 3) % cells
+    stmts = [Stmt([Access(0, W, (own,))], phase=const(p), loops=[Loop(0, hot)], name=f"w{p}")
+             for p in range(0, phases, 2)]
+    stmts += [Stmt([Access(0, R, (other,))], phase=const(p), guards=[tid.x % 3 - (1 if p % 2 == 0 else 0)],
+                   loops=[Loop(0, hot)], name=f"r{p}") for p in range(phases)]
+    return Model((blocks, 1, 1), (threads, 1, 1), [a], stmts, n_phases=phases, name=f"mix_{blocks}_{threads}_{cells}_{phases}")
+
+
+@pytest.mark.parametrize("phases", [1, 2, 7, 16])
+@pytest.mark.parametrize("blocks,threads", [(1, 1), (1, 33), (3, 96), (64, 256)])
+def test_candidates(rc, blocks, threads, phases):
+    check(rc, shared_mix(blocks, threads, max(1, threads), phases))
+    check(rc, shared_mix(blocks, threads, max(1, threads // 3), phases, scope=GLOBAL))
+
+
+def test_many_candidates_of_sixteen_intervals(rc):
+    # ~500 candidate cells and more per bucket: several windows of the table
+    check(rc, shared_mix(40, 512, 512, 16))
+
+
+@pytest.mark.parametrize("cells", [1, 3, 40])
+def test_hot_cells_exceed_the_registers(rc, cells):
+    # tens of thousands of keys in a few cells: a bucket read again in every step
+    check(rc, shared_mix(30, 200, cells, 4, hot=9))
+    check(rc, shared_mix(30, 200, cells, 1, scope=GLOBAL, hot=9))
+
+
+def word_model(block_extra):
+    """Interval, block, thread and kind fill exactly (or just exceed) 32 bits;
+    a few threads are left by the guards."""
+    blocks, threads = 1 << 17, 512        # 17 + 9 bits, kind 1, intervals 4 (32 phases would leave the path) + 1
+    a = Array("a", GLOBAL, (1 << (5 + block_extra),))
+    i = (tid.x + bid.x) % (1 << (5 + block_extra))
+    g = [const(3) - tid.x, const(40) - bid.x]
+    return Model((blocks << block_extra, 1, 1), (threads, 1, 1), [a],
+                 [Stmt([Access(0, W, (i,))], phase=const(15), guards=g),
+                  Stmt([Access(0, R, ((i + 1) % (1 << (5 + block_extra)),))], phase=const(0), guards=g)], n_phases=16,
+                 name=f"word{block_extra}")
+
+
+@pytest.mark.parametrize("extra", [0, 1])
+def test_key_word_widths(rc, extra):
+    m = word_model(extra)
+    h = rc.rc_model_create(m)
+    assert rc.rc_model_layout(h)["cell_shift"] == 31 + extra
+    check(rc, m)
+
+
+@pytest.mark.parametrize("n", [1, 31, 4320, 4321, 4700, 4701, 5120, 5121])
+def test_bucket_edges(rc, n):
+    a = Array("a", GLOBAL, (max(1, n // 2),))
+    m = Model((1, 1, 1), (1, 1, 1), [a], [Stmt([Access(0, W, (it(0) % max(1, n // 2),))], loops=[Loop(0, n)])])
+    check(rc, m)
+    m2 = Model((2, 1, 1), (1, 1, 1), [a], m.stmts)
+    check(rc, m2)
+
+
+@pytest.mark.parametrize("parts", [2, 16])
+def test_hash_parts_report_the_smallest_cell(rc, parts):
+    m = shared_mix(24, 128, 128, 5)
+    whole = rc.check(m)
+    got = [rc.check(m, {"part_count": parts, "part_index": i}) for i in range(parts)]
+    assert sum(r.racy_cells for r in got) == whole.racy_cells
+    assert min(r.witness for r in got if r.verdict) == whole.witness
