@@ -352,7 +352,7 @@ constexpr int kPartTileHost = kSortThreadsHost * 16;    // keys per tile of the 
 // buckets then cost less.
 constexpr uint32_t kFilterMaxSlotBits = 13;         // table slots of a bucket: 32 KB of 4-byte words
 constexpr uint32_t kFilterMaxLowBits = 32;          // (interval, block, thread, kind) bits: a table word
-constexpr uint64_t kFilterTarget = 4700;            // planned mean keys per bucket (at most)
+constexpr uint64_t kFilterTarget = 4600;            // planned mean keys per bucket (at most)
 constexpr uint64_t kFilterMinKeys = 512;            // ... and at least, where the cell bits ask for more buckets
 constexpr uint64_t kFilterOnePassKeys = 48 * 1024;  // ... and at most, where one partition pass does
 
@@ -407,7 +407,8 @@ struct Model {
   std::vector<uint8_t> program;   // host image of the uploaded program
   void* dev_program = nullptr;    // device allocation (program + unit offsets)
   size_t dev_bytes = 0;
-  uint64_t key_slots = 0;
+  uint64_t key_slots = 0;         // of all points (rc_expand_keys, the interpreted expansion)
+  uint64_t check_slots = 0;       // of a check: the generated expansion makes a key per distinct point
   uint64_t total_cells = 0;
   std::vector<uint64_t> array_base, array_cells;
   std::vector<uint32_t> array_shared;
@@ -476,8 +477,11 @@ struct CellFilter {
   uint64_t lo = 0, hi = ~0ull;
   uint64_t pmask = 0, pval = 0;
 };
+// all_points: every point of every nest in its slot (key_slots), not only the
+// distinct ones (check_slots)
 cudaError_t jit_expand_launch(const Model& m, uint64_t* keys, DevResult* res, cudaStream_t st,
-                              const CellFilter& cf = CellFilter(), const ExpandHist* eh = nullptr);
+                              const CellFilter& cf = CellFilter(), const ExpandHist* eh = nullptr,
+                              bool all_points = false);
 
 // implemented in lower.cpp
 rc_status lower_model(const rc_model_desc* d, Model* m, std::vector<int32_t>* general_stmt_ids);

@@ -214,7 +214,7 @@ void plan_workspace(const Model& m, const rc_check_opts* opts, WorkspacePlan* p)
     p->total = off;
     return;
   }
-  plan_workspace_keys(m, opts, n, m.host.cell_bits, p);
+  plan_workspace_keys(m, opts, m.check_slots, m.host.cell_bits, p);
 }
 
 bool bucket_path_allowed(uint32_t phase_bits, const rc_check_opts* opts) {
@@ -1652,7 +1652,7 @@ rc_status rc_model_create(const rc_model_desc* desc, rc_model** out) {
     delete mm;
     return RC_E_CUDA;
   }
-  m.key_slots = h.dense_slots + h.general_slots;
+  m.key_slots = m.check_slots = h.dense_slots + h.general_slots;
   // large models get a generated expansion kernel; failure keeps the interpreted one
   rc::jit_expand_build(&m);
   *out = mm;
@@ -2043,7 +2043,7 @@ rc_status rc_expand_keys(rc_model* mm, void* workspace, size_t ws_bytes, uint64_
   rc_status s = cuda_status(rc::launch_init_result(res, st));
   if (s != RC_OK) return s;
   if (m.jit_fn)
-    s = cuda_status(rc::jit_expand_launch(m, keys_dev, res, st));
+    s = cuda_status(rc::jit_expand_launch(m, keys_dev, res, st, rc::CellFilter(), nullptr, true));
   else
     s = cuda_status(rc::launch_expand(reinterpret_cast<const rc::DevModel*>(m.dev_program),
                                       m.host.n_stmts, m.host.n_threads, m.has_deep_loops, keys_dev, res, st));
