@@ -342,13 +342,15 @@ enum { RC_OPT_STAGE_TIMES = 1, RC_OPT_GRAPH = 2, RC_OPT_CHUNKED = 4, RC_OPT_LSD 
 /* Grouping step of the sort path.  By default a check (or a batch pack) whose
  * keys carry at most 16 barrier intervals groups its keys by cell with the
  * bucket path: two look-back-free partition passes on the top bits of a
- * bijective hash of the cell field, then a counting sort of every bucket in
- * shared memory on the hash's remaining bits, which leaves every cell's keys
- * together (cells in hash order), then the cell scan; its result is identical
- * to the radix-sorted check's.
+ * bijective hash of the cell, then, for models without warp or grid barriers
+ * whose cells have a table slot each in their bucket, the cell test in shared
+ * memory (also for up to 64 intervals when there are at least 2^16 keys), else a
+ * counting sort of every bucket in shared memory on the hash's remaining bits,
+ * which leaves every cell's keys together (cells in hash order), and the cell
+ * scan; the result is identical to the radix-sorted check's.
  * RC_OPT_LSD (or a non-zero digit_bits, or any test flag) selects the stable
- * LSD radix sort followed by the ordered scan instead; models of more than 16
- * intervals, chunked checks and rc_sort_keys always take that path. */
+ * LSD radix sort followed by the ordered scan instead; other models of more
+ * than 16 intervals, chunked checks and rc_sort_keys always take that path. */
 
 typedef struct rc_inst {
   uint64_t block;          /* linear block index bx + gx*(by + gy*bz)             */
@@ -495,9 +497,9 @@ typedef struct rc_stage_times {
   float histogram_ms;      /* digit histograms + digit offsets (bucket path: the
                               pass-A histogram and its offsets)                    */
   float sort_ms[16];       /* K2, one entry per pass (bucket path: partition
-                              passes A and B)                                      */
+                              passes A and B, then the cell test or local sort)    */
   uint32_t n_sort_passes;
-  float scan_ms;           /* K3 scan + fold (bucket path: the bucket fold)        */
+  float scan_ms;           /* K3 scan + fold (cell test: only its last step)       */
   float witness_ms;        /* K4 witness                                           */
   float total_ms;          /* from the first to the last event                     */
   uint64_t n_keys;         /* keys sorted and scanned                              */

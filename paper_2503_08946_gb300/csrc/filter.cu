@@ -1,6 +1,6 @@
-// The cell test of the bucket path for models without atomics and without warp
-// or grid barriers: every bucket's cells are decided in shared memory, without
-// sorting the bucket's keys.
+// The cell test of the bucket path for models without warp or grid barriers:
+// every bucket's cells are decided in shared memory, without sorting the
+// bucket's keys.
 //
 // A cell is racy iff it has a write and either two blocks meet in it or, inside
 // one block, some barrier interval holds two threads and a write (the
@@ -23,6 +23,14 @@
 // A representative decides exactly: if an interval (or cell) has a write and two
 // threads (or blocks), at least one of its keys differs from whichever write
 // was kept.  Which store wins does not matter, so the stores need no order.
+//
+// With atomics (AT; a 2-bit kind field) a conflict is a write, or an atomic and a
+// plain read.  The representative is then any write or atomic of the cell, and
+// beside the marks for blocks, threads and intervals the cell keeps whether it
+// has a write and a plain read, in all and in the representative's interval: two
+// blocks or threads meet in a conflict iff there is a write, or a read beside the
+// atomic (two threads among the atomics and reads of a group that holds both
+// always make an atomic and a read of different threads).
 //
 // What bounds it: one read of every key (8 bytes); about 78 warp instructions per
 // 32 keys keep the issue slots 76 % busy.  On the 4096 x 256 random affine model
@@ -65,14 +73,17 @@ __host__ __device__ __forceinline__ unsigned table_words(uint32_t r) {
 }
 __host__ __device__ __forceinline__ unsigned mask_words(uint32_t r) { return r < 5 ? 1u : (1u << (r - 5)); }
 // (four words behind the table: the slot of padding keys)
-size_t filter_smem(uint32_t r) { return ((size_t)table_words(r) + 4 + 5 * (size_t)mask_words(r) + 1) * sizeof(unsigned); }
+size_t filter_smem(uint32_t r, bool at) {
+  return ((size_t)table_words(r) + 4 + (at ? 10 : 5) * (size_t)mask_words(r) + 1 + (at ? 3 * table_words(r) / 32 : 0)) *
+         sizeof(unsigned);
+}
 
 // One block per bucket.  A bucket of at most kFltCap keys is held in registers
 // as (low word, slot); a larger one is read again in every step.  Key slots of
 // a thread past the bucket's end repeat its first key (the same instance, which
 // changes nothing), so no step tests for them; PAD: the bucket holds padding
 // keys (the unpartitioned single bucket), held as reads of the word behind the table.
-template <bool PAD, bool REGS>
+template <bool PAD, bool REGS, bool AT>
 __device__ __forceinline__ void filter_bucket(const FilterArgs& a, const uint64_t* src, uint64_t len) {
   extern __shared__ __align__(16) unsigned s_tab[];
   const unsigned tw = table_words(a.r), mw = mask_words(a.r);
@@ -81,13 +92,24 @@ __device__ __forceinline__ void filter_bucket(const FilterArgs& a, const uint64_
   unsigned* s_racy = s_wi + mw;         // racy cells
   unsigned* s_hot = s_racy + mw;        // racy candidate cells, a bit per candidate
   unsigned* s_rank = s_hot + mw + 1;    // candidate cells before each word of s_wi
+  // with atomics: cells with two threads in the representative's interval, with a
+  // write, with a read, and with those in its interval; the same three per entry
+  unsigned* s_g = s_rank + mw;
+  unsigned* s_w = s_g + mw;
+  unsigned* s_r = s_w + mw;
+  unsigned* s_wp = s_r + mw;
+  unsigned* s_rp = s_wp + mw;
+  unsigned* s_e2 = s_rp + mw;
+  unsigned* s_ew = s_e2 + tw / 32;
+  unsigned* s_er = s_ew + tw / 32;
   __shared__ unsigned s_wsum[kFltThreads / 32];
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
   const uint32_t pb = a.s.phase_bits, bb = a.s.block_bits, tb = a.s.thread_bits;
-  // a low word's fields: (block, thread), block, interval
-  const unsigned m_bt = (unsigned)(((1ull << (bb + tb)) - 1ull) << 1),
-                 m_b = (unsigned)(((1ull << bb) - 1ull) << (1 + tb)),
-                 m_p = (unsigned)(((1ull << pb) - 1ull) << (1 + tb + bb));
+  // a low word's fields: kind (R = 0, W = 1, A = 2), (block, thread), block, interval
+  constexpr unsigned kb = AT ? 2u : 1u, kmask = AT ? 3u : 1u;
+  const unsigned m_bt = (unsigned)(((1ull << (bb + tb)) - 1ull) << kb),
+                 m_b = (unsigned)(((1ull << bb) - 1ull) << (kb + tb)),
+                 m_p = (unsigned)(((1ull << pb) - 1ull) << (kb + tb + bb));
   const uint32_t cs = a.s.cell_shift;
   const unsigned smask = (1u << a.r) - 1u;
   const unsigned lmask = cs < 32 ? (1u << cs) - 1u : ~0u;
@@ -156,12 +178,12 @@ __device__ __forceinline__ void filter_bucket(const FilterArgs& a, const uint64_
   };
   // (the slots rounded up to whole 16-byte stores lie inside the table)
   clear_table(PAD ? tw + 4u : ((1u << a.r) + 3u) & ~3u);
-  for (unsigned i = tid; i < 4 * mw + 1; i += kFltThreads) s_two[i] = 0;
+  for (unsigned i = tid; i < (AT ? 10 : 4) * mw + 1; i += kFltThreads) s_two[i] = 0;
   __syncthreads();
-  // 1. the representative write of every written cell (a write's low word is odd)
+  // 1. the representative of every written cell (its low word is not 0)
   bool any = false;
   each([&](unsigned k, unsigned s) {
-    if (k & 1u) {
+    if (k & kmask) {
       s_tab[s] = k;
       any = true;
     }
@@ -172,7 +194,21 @@ __device__ __forceinline__ void filter_bucket(const FilterArgs& a, const uint64_
   each([&](unsigned k, unsigned s) {
     const unsigned rep = s_tab[s];
     const unsigned d = rep ^ k;
-    if (rep != 0u && (d & ((k & 1u) ? m_bt | m_p : m_bt)) != 0u) {
+    if constexpr (AT) {
+      if (rep == 0u) return;
+      const unsigned kind = k & kmask;
+      if (kind != 2u) mark(kind ? s_w : s_r, s);
+      any = any || (d & m_bt) != 0u;
+      if (d & m_b) {
+        mark(s_racy, s);   // (two blocks: racy if the cell has a conflict)
+      } else if (d & m_p) {
+        if (d & m_bt) mark(s_two, s);
+        if (kind) mark(s_wi, s);
+      } else {
+        if (d & m_bt) mark(s_g, s);
+        if (kind != 2u) mark(kind ? s_wp : s_rp, s);
+      }
+    } else if (rep != 0u && (d & ((k & 1u) ? m_bt | m_p : m_bt)) != 0u) {
       any = true;
       if (d & m_bt) mark((d & m_b) || !(d & m_p) ? s_racy : s_two, s);
       if ((k & 1u) && (d & m_p)) mark(s_wi, s);
@@ -183,7 +219,14 @@ __device__ __forceinline__ void filter_bucket(const FilterArgs& a, const uint64_
   // mask per thread
   unsigned cand = 0;
   if (tid < (int)mw) {
-    cand = s_two[tid] & s_wi[tid] & ~s_racy[tid];
+    if constexpr (AT) {
+      const unsigned conf = s_w[tid] | s_r[tid];
+      const unsigned racy = (s_racy[tid] & conf) | (s_g[tid] & (s_wp[tid] | s_rp[tid]));
+      s_racy[tid] = racy;
+      cand = s_wi[tid] & (s_two[tid] | s_g[tid]) & conf & ~racy;
+    } else {
+      cand = s_two[tid] & s_wi[tid] & ~s_racy[tid];
+    }
     s_wi[tid] = cand;
   }
   if (__syncthreads_or(cand != 0u)) {
@@ -209,15 +252,17 @@ __device__ __forceinline__ void filter_bucket(const FilterArgs& a, const uint64_
       if (PAD && s == tw) return ~0u;
       const unsigned m = s_wi[s >> 5];
       if (!((m >> (s & 31u)) & 1u)) return ~0u;
-      return ((s_rank[s >> 5] + __popc(m & ((1u << (s & 31u)) - 1u))) << pb) | (unsigned)((uint64_t)k >> (1 + bb + tb));
+      return ((s_rank[s >> 5] + __popc(m & ((1u << (s & 31u)) - 1u))) << pb) | (unsigned)((uint64_t)k >> (kb + bb + tb));
     };
     // windows of tw entries of the table
     for (unsigned e0 = 0; e0 < (ncand << pb); e0 += tw) {
       const unsigned used = min(tw, (ncand << pb) - e0);
       clear_table((used + 3u) & ~3u);
+      if constexpr (AT)
+        for (unsigned i = tid; i < 3 * (tw / 32); i += kFltThreads) s_e2[i] = 0;
       __syncthreads();
       each([&](unsigned k, unsigned s) {
-        if (k & 1u) {
+        if (k & kmask) {
           const unsigned e = entry(k, s) - e0;
           if (e < used) s_tab[e] = k;
         }
@@ -227,10 +272,22 @@ __device__ __forceinline__ void filter_bucket(const FilterArgs& a, const uint64_
         const unsigned e = entry(k, s) - e0;
         if (e < used) {
           const unsigned rep = s_tab[e];
-          if (rep != 0u && ((rep ^ k) & m_bt) != 0u) mark(s_hot, (e + e0) >> pb);
+          if constexpr (AT) {
+            if (rep == 0u) return;
+            if ((rep ^ k) & m_bt) mark(s_e2, e);
+            if ((k & kmask) != 2u) mark(k & kmask ? s_ew : s_er, e);
+          } else {
+            if (rep != 0u && ((rep ^ k) & m_bt) != 0u) mark(s_hot, (e + e0) >> pb);
+          }
         }
       });
       __syncthreads();
+      if constexpr (AT) {
+        for (unsigned i = tid; 32 * i < used; i += kFltThreads)
+          for (unsigned m = s_e2[i] & (s_ew[i] | s_er[i]); m; m &= m - 1u)
+            mark(s_hot, (32 * i + (unsigned)__ffs(m) - 1u + e0) >> pb);
+        __syncthreads();
+      }
     }
   }
   // the racy cells: counted, and the smallest by value kept.  Slot s of bucket b
@@ -273,27 +330,31 @@ __device__ __forceinline__ void filter_bucket(const FilterArgs& a, const uint64_
   }
 }
 
-template <bool PAD>
+template <bool PAD, bool AT>
 __global__ void __launch_bounds__(kFltThreads, kFltBlocks) bucket_filter_kernel(FilterArgs a) {
   const uint64_t lo = a.boff[blockIdx.x], hi = a.boff[blockIdx.x + 1];
   if (hi < lo + 2) return;              // a race needs two keys
-  if (hi - lo <= (uint64_t)kFltCap) filter_bucket<PAD, true>(a, a.keys_in + lo, hi - lo);
-  else filter_bucket<PAD, false>(a, a.keys_in + lo, hi - lo);
+  if (hi - lo <= (uint64_t)kFltCap) filter_bucket<PAD, true, AT>(a, a.keys_in + lo, hi - lo);
+  else filter_bucket<PAD, false, AT>(a, a.keys_in + lo, hi - lo);
+}
+
+template <bool PAD, bool AT>
+cudaError_t launch_filter(const FilterArgs& a, uint32_t D, cudaStream_t st) {
+  const cudaError_t e = ensure_kernel_smem(reinterpret_cast<const void*>(bucket_filter_kernel<PAD, AT>),
+                                           filter_smem(kFilterMaxSlotBits, AT));
+  if (e != cudaSuccess) return e;
+  bucket_filter_kernel<PAD, AT><<<1u << D, kFltThreads, filter_smem(a.r, AT), st>>>(a);
+  return cudaGetLastError();
 }
 
 }  // namespace
 
 cudaError_t launch_bucket_filter(const FilterArgs& a, uint32_t D, cudaStream_t st) {
   if (a.r > kFilterMaxSlotBits || a.s.cell_shift > kFilterMaxLowBits) return cudaErrorInvalidValue;
-  // an unpartitioned bucket holds padding keys, which take the table's last word
-  const bool pad = D == 0;
-  const void* fn = pad ? reinterpret_cast<const void*>(bucket_filter_kernel<true>)
-                       : reinterpret_cast<const void*>(bucket_filter_kernel<false>);
-  const cudaError_t e = ensure_kernel_smem(fn, filter_smem(kFilterMaxSlotBits));
-  if (e != cudaSuccess) return e;
-  if (pad) bucket_filter_kernel<true><<<1, kFltThreads, filter_smem(a.r), st>>>(a);
-  else bucket_filter_kernel<false><<<1u << D, kFltThreads, filter_smem(a.r), st>>>(a);
-  return cudaGetLastError();
+  // an unpartitioned bucket holds padding keys, which take the word behind the table
+  const bool at = a.s.thread_shift == 2;
+  if (D == 0) return at ? launch_filter<true, true>(a, D, st) : launch_filter<true, false>(a, D, st);
+  return at ? launch_filter<false, true>(a, D, st) : launch_filter<false, false>(a, D, st);
 }
 
 }  // namespace rc

@@ -354,6 +354,8 @@ constexpr uint32_t kFilterMaxSlotBits = 13;         // table slots of a bucket: 
 constexpr uint32_t kFilterMaxLowBits = 32;          // (interval, block, thread, kind) bits: a table word
 constexpr uint64_t kFilterTarget = 4600;            // planned mean keys per bucket (at most)
 constexpr uint64_t kFilterMinKeys = 512;            // ... and at least, where the cell bits ask for more buckets
+constexpr uint32_t kFilterMaxPhaseBits = 6;         // intervals: a bucket's candidates take a dozen tables at most
+constexpr uint64_t kFilterManyMinKeys = 1 << 16;    // fewest keys of a check of more than 16 intervals on this path
 constexpr uint64_t kFilterOnePassKeys = 48 * 1024;  // ... and at most, where one partition pass does
 
 struct BucketPlan {
@@ -372,9 +374,9 @@ struct BucketPlan {
 // host (runtime.cu): whether the bucket path applies to n keys of cb cell bits
 // (at most 2^kBucketMaxBits buckets of about kBucketTarget keys), its digit
 // widths, and its workspace section laid out from byte offset `off`
-// filter_ok: the model admits the table test (no atomics, no warp or grid
-// barriers, at most kFilterMaxLowBits key bits below the cell)
-bool plan_buckets(uint64_t n, uint64_t n_expect, uint32_t cb, bool filter_ok, size_t off, BucketPlan* bp);
+// filter_ok: the model admits the table test (no warp or grid barriers, at most kFilterMaxLowBits key bits below the cell)
+bool plan_buckets(uint64_t n, uint64_t n_expect, uint32_t cb, uint32_t phase_bits, bool filter_ok, size_t off,
+                  BucketPlan* bp);
 
 
 struct WorkspacePlan {
@@ -491,8 +493,8 @@ void plan_workspace(const Model& m, const rc_check_opts* opts, WorkspacePlan* p)
 // narrower sort of fewer bits, whose widest digit may be wider, fits it)
 void plan_workspace_keys(const Model& m, const rc_check_opts* opts, uint64_t n, uint32_t cell_bits, WorkspacePlan* p,
                          uint32_t min_lookback_bits = 0, bool allow_bucket = true);
-// whether options and a key layout of phase_bits phase bits admit the bucket path
-bool bucket_path_allowed(uint32_t phase_bits, const rc_check_opts* opts);
+// whether the options admit the bucket path
+bool bucket_path_allowed(const rc_check_opts* opts);
 void plan_sort(uint32_t lo, uint32_t hi, uint32_t digit_bits, SortPlan* sp);
 uint32_t bit_length(uint64_t v);
 

@@ -217,15 +217,14 @@ void plan_workspace(const Model& m, const rc_check_opts* opts, WorkspacePlan* p)
   plan_workspace_keys(m, opts, m.check_slots, m.host.cell_bits, p);
 }
 
-bool bucket_path_allowed(uint32_t phase_bits, const rc_check_opts* opts) {
-  if (phase_bits > kScanTablePhaseBits) return false;   // the fold keeps per-interval masks of 16 intervals
+bool bucket_path_allowed(const rc_check_opts* opts) {
   if (opts && ((opts->flags & RC_OPT_LSD) || opts->digit_bits || opts->test_flags)) return false;
   return true;
 }
 
 // whether a model (or a batch pack) admits the cell test in shared memory
-static bool filter_allowed(bool atomics_or_scopes, uint32_t cell_shift) {
-  return !atomics_or_scopes && cell_shift <= kFilterMaxLowBits;
+static bool filter_allowed(bool sync_scopes, uint32_t cell_shift) {
+  return !sync_scopes && cell_shift <= kFilterMaxLowBits;
 }
 
 // n key slots, of which about n_expect are kept (a hash-partitioned check keeps
@@ -247,12 +246,18 @@ static uint32_t filter_bucket_bits(uint64_t n_expect, uint32_t cb) {
   return D;
 }
 
-bool plan_buckets(uint64_t n, uint64_t n_expect, uint32_t cb, bool filter_ok, size_t off, BucketPlan* bp) {
+bool plan_buckets(uint64_t n, uint64_t n_expect, uint32_t cb, uint32_t phase_bits, bool filter_ok, size_t off,
+                  BucketPlan* bp) {
   *bp = BucketPlan();
   if (n == 0 || n >= (1ull << 32) || cb == 0 || cb > 62) return false;
+  // more than 16 intervals: the cell test only (the scan keeps masks of 16), where
+  // its candidates' intervals fit a few tables and there are keys to move
+  const bool many = phase_bits > kScanTablePhaseBits;
+  if (many && (phase_bits > kFilterMaxPhaseBits || n < kFilterManyMinKeys)) return false;
   if (n_expect == 0 || n_expect > n) n_expect = n;
   uint32_t D = filter_ok ? filter_bucket_bits(n_expect, cb) : ~0u;
   bp->filter = D != ~0u;
+  if (!bp->filter && many) return false;
   if (!bp->filter) {
     D = 0;
     while (D < cb && D < kBucketMaxBits && (n_expect >> D) > kBucketTarget) ++D;
@@ -318,10 +323,9 @@ void plan_workspace_keys(const Model& m, const rc_check_opts* opts, uint64_t n, 
   const bool part = opts && opts->part_count > 1;
   const uint32_t part_bits = part ? bit_length(opts->part_count - 1) : 0u;
   const uint64_t n_expect = part ? n / opts->part_count + n / (16ull * opts->part_count) + 1 : n;
-  if (allow_bucket && bucket_path_allowed(m.host.phase_bits, opts) && cell_bits > part_bits &&
-      plan_buckets(n, n_expect, cell_bits - part_bits,
-                   filter_allowed(m.has_atomic || m.sync_scopes, m.host.cell_shift), off,
-                   &p->bucket)) {
+  if (allow_bucket && bucket_path_allowed(opts) && cell_bits > part_bits &&
+      plan_buckets(n, n_expect, cell_bits - part_bits, m.host.phase_bits,
+                   filter_allowed(m.sync_scopes, m.host.cell_shift), off, &p->bucket)) {
     // the bucket path: its own section instead of the radix-sort sections
     p->zero_lo = p->bucket.zero_lo;
     p->zero_hi = p->bucket.zero_hi;
@@ -1192,9 +1196,8 @@ rc_status plan_batch(rc_model* const* models, size_t n, const rc_check_opts* opt
     o = align256(o + k.n_keys * 8);
     p.keys_off[1] = o;
     o = align256(o + k.n_keys * 8);
-    if (rc::bucket_path_allowed(k.pb, opts) && rc::plan_buckets(k.n_keys, k.n_keys, k.cell_bits,
-                                                               rc::filter_allowed(k.kb != 1 || k.sy, ps + k.pb), o,
-                                                               &p.bucket)) {
+    if (rc::bucket_path_allowed(opts) &&
+        rc::plan_buckets(k.n_keys, k.n_keys, k.cell_bits, k.pb, rc::filter_allowed(k.sy, ps + k.pb), o, &p.bucket)) {
       p.zero_lo = p.bucket.zero_lo;
       p.zero_hi = p.bucket.zero_hi;
       o = p.bucket.end;

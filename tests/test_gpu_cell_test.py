@@ -7,7 +7,8 @@ import pytest
 
 import oracle
 import workloads as w
-from workloads.spec import Access, Array, GLOBAL, Loop, Model, R, SHARED, Stmt, W, bid, const, it, tid
+from workloads.rng import SplitMix64
+from workloads.spec import A, Access, Array, GLOBAL, Loop, Model, R, SHARED, Stmt, W, bid, const, it, tid
 
 pytestmark = pytest.mark.gpu
 
@@ -95,3 +96,42 @@ def test_hash_parts_report_the_smallest_cell(rc, parts):
     got = [rc.check(m, {"part_count": parts, "part_index": i}) for i in range(parts)]
     assert sum(r.racy_cells for r in got) == whole.racy_cells
     assert min(r.witness for r in got if r.verdict) == whole.witness
+
+
+def atomic_mix(seed, blocks, threads, cells, phases, scope):
+    """Reads, writes and atomics of few cells in few (or many) intervals, each
+    statement by a part of the threads and blocks: every combination of kinds in
+    a cell, an interval and a block turns up over the seeds."""
+    rng = SplitMix64(0xA70 ^ seed * 0x9E3779B97F4A7C15)
+    a = Array("a", scope, (cells,))
+    stmts = []
+    for s in range(rng.uniform_int(2, 9)):
+        kind = (R, A, A, W)[rng.below(4)]
+        i = (rng.uniform_int(0, 3) * tid.x + rng.uniform_int(0, 2) * bid.x + rng.below(cells)) % cells
+        guards = [rng.below(threads) - tid.x] if rng.chance(0.5) else [rng.uniform_int(0, 2) - tid.x % 3]
+        if rng.chance(0.3):
+            guards.append(const(0) - bid.x % 2)
+        stmts.append(Stmt([Access(0, kind, (i,))], phase=const(rng.below(phases)), guards=guards, name=f"{kind}{s}"))
+    return Model((blocks, 1, 1), (threads, 1, 1), [a], stmts, n_phases=phases, name=f"amix{seed}")
+
+
+@pytest.mark.parametrize("seed", range(60))
+def test_atomics(rc, seed):
+    scope = (SHARED, GLOBAL)[seed & 1]
+    check(rc, atomic_mix(seed, 1 + seed % 3, 40, 1 + seed % 13, 1 + seed % 5, scope))
+    check(rc, atomic_mix(seed, 3, 64, 64 if scope == SHARED else 700, 16, scope))
+
+
+@pytest.mark.parametrize("seed", range(8))
+def test_atomics_partitioned(rc, seed):
+    check(rc, atomic_mix(100 + seed, 60, 256, 200, 1 + seed, (SHARED, GLOBAL)[seed & 1]))
+
+
+@pytest.mark.parametrize("phases", [17, 32, 33, 64, 65])
+def test_many_intervals(rc, phases):
+    m = shared_mix(20, 192, 100, phases)          # 65,280 key slots and more at 17 intervals and more
+    n = rc.rc_model_layout(rc.rc_model_create(m))["key_slots"]
+    assert n >= 65536 or phases == 17
+    check(rc, m)
+    check(rc, atomic_mix(7, 300, 256, 50, phases, SHARED))
+    check(rc, atomic_mix(8, 300, 256, 3000, phases, GLOBAL))
