@@ -171,6 +171,44 @@ __global__ void __launch_bounds__(1024) bucket_scan_a_kernel(BucketArgs a) {
   }
 }
 
+// Bucket offsets and pass-B cursors: the buckets of an A-bucket begin at its
+// offset, so every A-bucket scans its own 2^dB counts (one block each, four
+// counts a thread at most).
+__global__ void __launch_bounds__(256) bucket_scan_b_kernel(BucketArgs a) {
+  const unsigned nb = 1u << a.dB;
+  const uint64_t b0 = (uint64_t)blockIdx.x << a.dB;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  __shared__ unsigned long long wsum[8];
+  constexpr int kPer = (1 << kBucketMaxDigitBits) / 256;
+  unsigned long long v[kPer], s = 0;
+#pragma unroll
+  for (int i = 0; i < kPer; ++i) {
+    const unsigned d = threadIdx.x * kPer + i;
+    v[i] = d < nb ? a.hist_b[b0 + d] : 0ull;
+    s += v[i];
+  }
+  unsigned long long x = s;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const unsigned long long y = __shfl_up_sync(FULL, x, o);
+    if (lane >= o) x += y;
+  }
+  if (lane == 31) wsum[w] = x;
+  __syncthreads();
+  unsigned long long run = a.off_a[blockIdx.x] + x - s;
+  for (int i = 0; i < w; ++i) run += wsum[i];
+#pragma unroll
+  for (int i = 0; i < kPer; ++i) {
+    const unsigned d = threadIdx.x * kPer + i;
+    if (d < nb) {
+      a.boff[b0 + d] = run;
+      a.cur_b[b0 + d] = run;
+    }
+    run += v[i];
+  }
+  if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) a.boff[(uint64_t)gridDim.x << a.dB] = a.off_a[gridDim.x];
+}
+
 __global__ void bucket_whole_kernel(unsigned long long* boff, uint64_t n) {
   boff[0] = 0;
   boff[1] = n;
@@ -666,11 +704,7 @@ __global__ void bucket_finish_kernel(FinishArgs fa) {
   if (i >= nr) return;
   DevResult* r = fa.res + i;
   const unsigned long long c = r->hash_cell;
-  if (c == ~0ull) return;
-  const uint64_t b = fa.D ? (cell_hash_of(c, fa.cmask) >> (fa.cb - fa.D)) : 0ull;
-  r->min_start = fa.boff[b];
-  r->seg_end = fa.boff[b + 1];
-  r->cell = c;
+  if (c != ~0ull) bucket_of_racy_cell(fa, r, c);
 }
 
 }  // namespace
@@ -701,12 +735,8 @@ cudaError_t launch_bucket_hist_b(const BucketArgs& a, uint64_t tiles_h, cudaStre
 }
 
 cudaError_t launch_bucket_scan_b(const BucketArgs& a, cudaStream_t st) {
-  const uint64_t nb = 1ull << (a.dA + a.dB);
-  cudaError_t e = scan_u64_exclusive(reinterpret_cast<const uint64_t*>(a.hist_b), reinterpret_cast<uint64_t*>(a.boff),
-                                     nb, 0, reinterpret_cast<uint64_t*>(a.temp),
-                                     reinterpret_cast<uint64_t*>(a.boff + nb), st);
-  if (e != cudaSuccess) return e;
-  return cudaMemcpyAsync(a.cur_b, a.boff, nb * 8, cudaMemcpyDeviceToDevice, st);
+  bucket_scan_b_kernel<<<1u << a.dA, 256, 0, st>>>(a);
+  return cudaGetLastError();
 }
 
 cudaError_t launch_bucket_pass_b(const BucketArgs& a, uint64_t tiles_b, cudaStream_t st) {

@@ -162,7 +162,6 @@ struct BucketArgs {
   unsigned long long* hist_b;       // [2^D] keys per bucket
   unsigned long long* boff;         // [2^D + 1] bucket offsets
   unsigned long long* cur_b;        // [2^D] pass-B output cursors
-  unsigned long long* temp;         // scan scratch
   unsigned int* err;
 };
 cudaError_t launch_bucket_hist_a(const BucketArgs& a, cudaStream_t st);
@@ -263,6 +262,20 @@ struct FinishArgs {
   uint32_t cb, D;
 };
 cudaError_t launch_bucket_finish(const FinishArgs& a, cudaStream_t st);
+#ifdef __CUDACC__
+__device__ __forceinline__ void bucket_of_racy_cell(const FinishArgs& fa, DevResult* r, unsigned long long cell) {
+  const uint64_t b = fa.D ? (((uint64_t)cell * kCellHashMul) & fa.cmask) >> (fa.cb - fa.D) : 0ull;
+  r->min_start = fa.boff[b];
+  r->seg_end = fa.boff[b + 1];
+  r->cell = cell;
+}
+#endif
+// scan.cu: that and the witness steps over the bucket (a.keys)
+cudaError_t launch_bucket_witness(const ScanArgs& a, const FinishArgs& fa, cudaStream_t st);
+// scan.cu: the start of a check: n result records, one more (or null), the cleared
+// range, a work queue (or null)
+cudaError_t launch_init_check(DevResult* res, uint32_t n, DevResult* more, void* zero, size_t zero_bytes,
+                              unsigned long long* queue, cudaStream_t st);
 cudaError_t launch_init_result(DevResult* res, cudaStream_t st, uint32_t n = 1);
 uint64_t scan_long_capacity(uint64_t n, uint32_t n_warps);
 

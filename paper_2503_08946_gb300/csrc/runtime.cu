@@ -296,8 +296,6 @@ bool plan_buckets(uint64_t n, uint64_t n_expect, uint32_t cb, uint32_t phase_bit
   off = align256(off + (nb + 1) * 8);
   bp->cur_b = off;
   off = align256(off + nb * 8);
-  bp->temp = off;
-  off = align256(off + scan_u64_temp_bytes(nb));
   bp->end = off;
   return true;
 }
@@ -456,7 +454,7 @@ rc_status enqueue_sort(const rc::WorkspacePlan& p, uint8_t* ws, uint64_t* buf0, 
 // return *final_keys is the buffer the witness reads.  Stage events: after the
 // pass-A histogram (i_hist), around each pass, around the pass-B histogram.
 rc_status enqueue_bucketed(const rc::WorkspacePlan& p, uint8_t* ws, uint64_t* buf0, uint64_t* buf1,
-                           const rc::ScanArgs& sa, cudaStream_t st, const uint64_t** final_keys,
+                           const rc::ScanArgs& sa, cudaStream_t st, const uint64_t** final_keys, rc::FinishArgs* fin_args,
                            rc_ticket_s* timed = nullptr, bool hist_a_done = false, uint32_t cell_bits = 0,
                            uint32_t part_index = 0) {
   const rc::BucketPlan& bp = p.bucket;
@@ -479,7 +477,6 @@ rc_status enqueue_bucketed(const rc::WorkspacePlan& p, uint8_t* ws, uint64_t* bu
   a.hist_b = u64(bp.hist_b);
   a.boff = u64(bp.boff);
   a.cur_b = u64(bp.cur_b);
-  a.temp = u64(bp.temp);
   a.err = sa.err;
   uint64_t* fin = buf0;
   uint64_t* scratch = buf1;
@@ -514,7 +511,7 @@ rc_status enqueue_bucketed(const rc::WorkspacePlan& p, uint8_t* ws, uint64_t* bu
     }
   }
   if (s != RC_OK) return s;
-  rc::FinishArgs fa;
+  rc::FinishArgs& fa = *fin_args;
   fa.res = sa.res;
   fa.n_models = sa.n_models;
   fa.boff = a.boff;
@@ -534,7 +531,6 @@ rc_status enqueue_bucketed(const rc::WorkspacePlan& p, uint8_t* ws, uint64_t* bu
     s = cuda_status(rc::launch_bucket_filter(f, bp.D, st));
     if (tm) { timed->i_pass_from[n_pass] = tm->n - 1; timed->i_pass_to[n_pass] = tm->n; tm->mark(); }
     ++n_pass;
-    if (s == RC_OK) s = cuda_status(rc::launch_bucket_finish(fa, st));
     if (timed) {
       timed->n_pass = n_pass;
       timed->bucketed = true;
@@ -566,7 +562,6 @@ rc_status enqueue_bucketed(const rc::WorkspacePlan& p, uint8_t* ws, uint64_t* bu
   sc.by_cell = 1;
   sc.phase_table = 1;
   if (s == RC_OK) s = cuda_status(rc::launch_scan(sc, st));
-  if (s == RC_OK) s = cuda_status(rc::launch_bucket_finish(fa, st));
   if (timed) {
     timed->n_pass = n_pass;
     timed->bucketed = true;
@@ -598,9 +593,10 @@ rc_status enqueue_check(rc_model* model, const rc_check_opts* opts, uint8_t* ws,
     timed->n_keys = p.n_keys;
   }
   const rc::DevModel* dm = reinterpret_cast<const rc::DevModel*>(m.dev_program);
-  rc_status s = cuda_status(rc::launch_init_result(res, st));
-  if (s != RC_OK) return s;
+  rc_status s = RC_OK;
   if (p.hash) {
+    s = cuda_status(rc::launch_init_result(res, st));
+    if (s != RC_OK) return s;
     rc::HashArgs h;
     h.gkey = reinterpret_cast<unsigned long long*>(ws + p.gkey_off);
     h.gword = reinterpret_cast<unsigned long long*>(ws + p.gword_off);
@@ -638,7 +634,7 @@ rc_status enqueue_check(rc_model* model, const rc_check_opts* opts, uint8_t* ws,
       s = cuda_status(cudaMemcpyAsync(host_out, res, sizeof(rc::DevResult), cudaMemcpyDeviceToHost, st));
     return s;
   }
-  s = cuda_status(cudaMemsetAsync(ws + p.zero_lo, 0, p.zero_hi - p.zero_lo, st));
+  s = cuda_status(rc::launch_init_check(res, 1, nullptr, ws + p.zero_lo, p.zero_hi - p.zero_lo, nullptr, st));
   if (s != RC_OK) return s;
   if (tm) { timed->i_start = tm->n; tm->mark(); }
   // the bucket path's pass-A histogram is counted by the generated expansion
@@ -681,14 +677,15 @@ rc_status enqueue_check(rc_model* model, const rc_check_opts* opts, uint8_t* ws,
   if (p.bucket.on) {
     // the bucket path: partition passes and the bucket fold
     const uint64_t* fin = nullptr;
+    rc::FinishArgs fa;
     rc::ScanArgs sa = scan_args(m, p, ws, 0);
     s = enqueue_bucketed(p, ws, reinterpret_cast<uint64_t*>(ws + p.keys_off[0]),
-                         reinterpret_cast<uint64_t*>(ws + p.keys_off[1]), sa, st, &fin, timed, fuse_hist, m.host.cell_bits,
+                         reinterpret_cast<uint64_t*>(ws + p.keys_off[1]), sa, st, &fin, &fa, timed, fuse_hist, m.host.cell_bits,
                          opts ? opts->part_index : 0u);
     if (s != RC_OK) return s;
     if (tm) { timed->i_scan = tm->n; tm->mark(); }
     sa.keys = fin;
-    s = cuda_status(rc::launch_witness(sa, st));
+    s = cuda_status(rc::launch_bucket_witness(sa, fa, st));
     if (s != RC_OK) return s;
     if (tm) { timed->i_wit = tm->n; tm->mark(); }
     if (host_out) s = cuda_status(cudaMemcpyAsync(host_out, res, sizeof(rc::DevResult), cudaMemcpyDeviceToHost, st));
@@ -1295,14 +1292,15 @@ rc_status enqueue_batch_device(const BatchLayout& L, size_t n, const rc_check_op
   auto* queue = reinterpret_cast<unsigned long long*>(ws + L.queue_off);
   const uint64_t spin = (opts && opts->spin_limit) ? opts->spin_limit : (1ull << 20);
   rc_status s = cuda_status(cudaMemcpyAsync(ws + L.table_off, upload, L.upload_bytes, cudaMemcpyHostToDevice, st));
-  if (s == RC_OK) s = cuda_status(rc::launch_init_result(res, st, (uint32_t)n));
+  bool first = true;
   for (const BatchPack& k : L.packs) {
     if (s != RC_OK) break;
     const rc::WorkspacePlan& p = k.p;
     const uint32_t nm = (uint32_t)(k.i1 - k.i0);
-    s = cuda_status(rc::launch_init_result(pres, st));
-    if (s == RC_OK) s = cuda_status(cudaMemsetAsync(ws + p.zero_lo, 0, p.zero_hi - p.zero_lo, st));
-    if (s == RC_OK) s = cuda_status(cudaMemsetAsync(queue, 0, 8, st));
+    // (the first pack's start initialises every model's record)
+    s = cuda_status(rc::launch_init_check(res, first ? (uint32_t)n : 0u, pres, ws + p.zero_lo, p.zero_hi - p.zero_lo,
+                                          queue, st));
+    first = false;
     if (s != RC_OK) break;
     rc::BatchArgs ba;
     ba.models = dtable + k.i0;
@@ -1351,13 +1349,15 @@ rc_status enqueue_batch_device(const BatchLayout& L, size_t n, const rc_check_op
     sa.grid_of = k.grid_of;
     if (p.bucket.on) {
       const uint64_t* fin = nullptr;
+      rc::FinishArgs fa;
       s = enqueue_bucketed(p, ws, reinterpret_cast<uint64_t*>(ws + p.keys_off[0]),
-                           reinterpret_cast<uint64_t*>(ws + p.keys_off[1]), sa, st, &fin, nullptr, false, k.cell_bits);
+                           reinterpret_cast<uint64_t*>(ws + p.keys_off[1]), sa, st, &fin, &fa, nullptr, false, k.cell_bits);
       sa.keys = fin;
+      if (s == RC_OK) s = cuda_status(rc::launch_bucket_witness(sa, fa, st));
     } else {
       s = cuda_status(rc::launch_scan(sa, st));
+      if (s == RC_OK) s = cuda_status(rc::launch_witness(sa, st));
     }
-    if (s == RC_OK) s = cuda_status(rc::launch_witness(sa, st));
     if (s == RC_OK) s = cuda_status(rc::launch_batch_errors(pres, res + k.i0, nm, st));
   }
   return s;

@@ -33,7 +33,10 @@
 //      smallest instance that has a partner (x), and x's smallest partner (y).
 //      The smallest participating instance always lies in the lowest block of a
 //      racy cell, so only that block's phase groups are needed.
+#include <cooperative_groups.h>
 #include <cuda_runtime.h>
+
+#include <algorithm>
 
 #include "fold.cuh"
 #include "kernels.h"
@@ -1077,6 +1080,11 @@ __global__ void __launch_bounds__(kLongThreads) scan_long_table_kernel(ScanArgs 
   }
 }
 
+// Blocks of the witness of one check: a cluster reads a bucket of the checks that
+// take it (at most kWitnessClusterKeys key slots) faster than five launches take.
+constexpr int kWitnessCluster = 8;
+constexpr uint64_t kWitnessClusterKeys = 1ull << 24;
+
 // One warp per result: the end of its first racy cell.
 __global__ void scan_finish_kernel(ScanArgs a) {
   DevResult* r = a.res + blockIdx.x;
@@ -1125,10 +1133,14 @@ __device__ __forceinline__ bool kinds_conflict(unsigned kx, unsigned ky) {
 // block's).  With several grid intervals the lowest block's instances may all
 // be ordered before the racing ones, so every block keeps its records.
 constexpr unsigned kGroupWords = kWitnessGroupWords;
-// Each kernel handles result blockIdx.y (one per model of a batch) with the
-// blocks of its x dimension.
-__device__ __forceinline__ unsigned* groups_of(const ScanArgs& a) {
-  return a.groups + (size_t)blockIdx.y * kGroupWords * ((size_t)1 << (a.phase_bits + a.wit_block_bits));
+// Each step handles result mi (one per model of a batch) with nb blocks, of
+// which this one is number bi.  What an earlier step wrote is read past L1
+// (__ldcg), since the steps may share one kernel.
+struct WitnessBlock {
+  uint32_t mi, bi, nb;
+};
+__device__ __forceinline__ unsigned* groups_of(const ScanArgs& a, const WitnessBlock& wb) {
+  return a.groups + (size_t)wb.mi * kGroupWords * ((size_t)1 << (a.phase_bits + a.wit_block_bits));
 }
 // the record of (block b, fine interval q)
 __device__ __forceinline__ unsigned* group_rec(const ScanArgs& a, unsigned* groups, unsigned b, unsigned q) {
@@ -1142,13 +1154,13 @@ __device__ __forceinline__ const unsigned* group_rec(const ScanArgs& a, const un
 }
 
 // the cell summary: blocks of all instances and of each kind
-__global__ void __launch_bounds__(256) witness_cell_kernel(ScanArgs a) {
-  DevResult* r = a.res + blockIdx.y;
-  const uint64_t s = r->min_start;
+__device__ __forceinline__ void witness_cell(const ScanArgs& a, const WitnessBlock wb) {
+  DevResult* r = a.res + wb.mi;
+  const uint64_t s = __ldcg(&r->min_start);
   const uint32_t n_groups = 1u << (a.phase_bits + a.wit_block_bits);
-  unsigned* groups = groups_of(a);
+  unsigned* groups = groups_of(a, wb);
   if (s == ~0ull) return;
-  for (uint32_t g = blockIdx.x * blockDim.x + threadIdx.x; g < n_groups; g += gridDim.x * blockDim.x) {
+  for (uint32_t g = wb.bi * blockDim.x + threadIdx.x; g < n_groups; g += wb.nb * blockDim.x) {
     unsigned* gr = groups + g * kGroupWords;
     gr[0] = 0xffffffffu;
     gr[1] = 0;
@@ -1160,11 +1172,11 @@ __global__ void __launch_bounds__(256) witness_cell_kernel(ScanArgs a) {
       gr[12 + 2 * k] = 0;
     }
   }
-  const uint64_t e = r->seg_end;
-  const uint64_t wcell = r->cell;
+  const uint64_t e = __ldcg(&r->seg_end);
+  const uint64_t wcell = __ldcg(&r->cell);
   unsigned minb = 0xffffffffu, maxb = 0;
   unsigned kmin[3] = {0xffffffffu, 0xffffffffu, 0xffffffffu}, kmax[3] = {0, 0, 0}, kany[3] = {0, 0, 0};
-  for (uint64_t i = s + blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < e; i += (uint64_t)gridDim.x * blockDim.x) {
+  for (uint64_t i = s + wb.bi * (uint64_t)blockDim.x + threadIdx.x; i < e; i += (uint64_t)wb.nb * blockDim.x) {
     const uint64_t key = a.keys[i];
     if ((key >> a.cell_shift) != wcell) continue;   // the bucket path's range holds other cells too
     const Fields f = fields(a, key);
@@ -1201,16 +1213,16 @@ __global__ void __launch_bounds__(256) witness_cell_kernel(ScanArgs a) {
   }
 }
 
-__global__ void __launch_bounds__(256) witness_group_kernel(ScanArgs a) {
-  DevResult* r = a.res + blockIdx.y;
-  const SyncTabs syt = sync_tabs_of(a, blockIdx.y);
-  unsigned* groups = groups_of(a);
-  const uint64_t s = r->min_start;
+__device__ __forceinline__ void witness_group(const ScanArgs& a, const WitnessBlock wb) {
+  DevResult* r = a.res + wb.mi;
+  const SyncTabs syt = sync_tabs_of(a, wb.mi);
+  unsigned* groups = groups_of(a, wb);
+  const uint64_t s = __ldcg(&r->min_start);
   if (s == ~0ull) return;
-  const uint64_t e = r->seg_end;
-  const uint64_t wcell = r->cell;
-  const unsigned b0 = r->minb;
-  for (uint64_t i = s + blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < e; i += (uint64_t)gridDim.x * blockDim.x) {
+  const uint64_t e = __ldcg(&r->seg_end);
+  const uint64_t wcell = __ldcg(&r->cell);
+  const unsigned b0 = __ldcg(&r->minb);
+  for (uint64_t i = s + wb.bi * (uint64_t)blockDim.x + threadIdx.x; i < e; i += (uint64_t)wb.nb * blockDim.x) {
     const uint64_t key = a.keys[i];
     if ((key >> a.cell_shift) != wcell) continue;   // the bucket path's range holds other cells too
     const Fields f = fields(a, key);
@@ -1231,20 +1243,21 @@ __global__ void __launch_bounds__(256) witness_group_kernel(ScanArgs a) {
   }
 }
 
-__global__ void __launch_bounds__(256) witness_x_kernel(ScanArgs a) {
-  DevResult* r = a.res + blockIdx.y;
-  const SyncTabs syt = sync_tabs_of(a, blockIdx.y);
-  const unsigned* groups = groups_of(a);
-  const uint64_t s = r->min_start;
+__device__ __forceinline__ void witness_x(const ScanArgs& a, const WitnessBlock wb) {
+  DevResult* r = a.res + wb.mi;
+  const SyncTabs syt = sync_tabs_of(a, wb.mi);
+  const unsigned* groups = groups_of(a, wb);
+  const uint64_t s = __ldcg(&r->min_start);
   if (s == ~0ull) return;
-  const uint64_t e = r->seg_end;
-  const uint64_t wcell = r->cell;
-  const unsigned b0 = r->minb;
-  const unsigned kminb[3] = {r->minRb, r->minWb, r->minAb}, kmaxb[3] = {r->maxRb, r->maxWb, r->maxAb};
-  const unsigned kany[3] = {r->anyR, r->anyW, r->anyA};
+  const uint64_t e = __ldcg(&r->seg_end);
+  const uint64_t wcell = __ldcg(&r->cell);
+  const unsigned b0 = __ldcg(&r->minb);
+  const unsigned kminb[3] = {__ldcg(&r->minRb), __ldcg(&r->minWb), __ldcg(&r->minAb)},
+                 kmaxb[3] = {__ldcg(&r->maxRb), __ldcg(&r->maxWb), __ldcg(&r->maxAb)};
+  const unsigned kany[3] = {__ldcg(&r->anyR), __ldcg(&r->anyW), __ldcg(&r->anyA)};
   const uint32_t kb = a.thread_shift;
   unsigned long long best = ~0ull;
-  for (uint64_t i = s + blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < e; i += (uint64_t)gridDim.x * blockDim.x) {
+  for (uint64_t i = s + wb.bi * (uint64_t)blockDim.x + threadIdx.x; i < e; i += (uint64_t)wb.nb * blockDim.x) {
     const uint64_t key = a.keys[i];
     if ((key >> a.cell_shift) != wcell) continue;   // the bucket path's range holds other cells too
     const Fields f = fields(a, key);
@@ -1258,7 +1271,7 @@ __global__ void __launch_bounds__(256) witness_x_kernel(ScanArgs a) {
       if (!kinds_conflict(f.k, (unsigned)k)) continue;
       // a conflicting instance of another thread in the same block and (fine) phase
       const unsigned* gk = g + 2 + 3 * k;
-      same |= gk[2] && (gk[0] != f.t || gk[1] != f.t);
+      same |= __ldcg(gk + 2) && (__ldcg(gk) != f.t || __ldcg(gk + 1) != f.t);
       if (!syt.on) {
         // a conflicting instance in another block (global cells; a shared cell has one block)
         cross |= kany[k] && (kminb[k] != b0 || kmaxb[k] != b0);
@@ -1270,12 +1283,12 @@ __global__ void __launch_bounds__(256) witness_x_kernel(ScanArgs a) {
       for (unsigned q = 0; q < (1u << a.phase_bits); ++q) {
         const unsigned* gq = group_rec(a, groups, 0u, q);
         // (a record with a key of kind k: q is a fine interval of the model)
-        if (gq[11 + 2 * k] != 0xffffffffu && (gq[11 + 2 * k] != xb || gq[12 + 2 * k] != xb) &&
-            grid_q(a, syt, q) == xg)
+        const unsigned q0 = __ldcg(gq + 11 + 2 * k), q1 = __ldcg(gq + 12 + 2 * k);
+        if (q0 != 0xffffffffu && (q0 != xb || q1 != xb) && grid_q(a, syt, q) == xg)
           cross = true;
         if (q != f.p && coarse_q(syt, q) == xc) {
           const unsigned* gqk = group_rec(a, groups, xb, q) + 2 + 3 * k;
-          if (gqk[2] && ((gqk[0] >> 5) != (f.t >> 5) || (gqk[1] >> 5) != (f.t >> 5))) same = true;
+          if (__ldcg(gqk + 2) && ((__ldcg(gqk) >> 5) != (f.t >> 5) || (__ldcg(gqk + 1) >> 5) != (f.t >> 5))) same = true;
         }
       }
     }
@@ -1299,25 +1312,25 @@ __global__ void __launch_bounds__(256) witness_x_kernel(ScanArgs a) {
   if ((threadIdx.x & 31) == 0 && best != ~0ull) atomicMin(&r->x_rank, best);
 }
 
-__global__ void __launch_bounds__(256) witness_y_kernel(ScanArgs a) {
-  DevResult* r = a.res + blockIdx.y;
-  const SyncTabs syt = sync_tabs_of(a, blockIdx.y);
-  const uint64_t s = r->min_start;
-  if (s == ~0ull || r->x_rank == ~0ull) return;
-  const uint64_t e = r->seg_end;
-  const uint64_t wcell = r->cell;
+__device__ __forceinline__ void witness_y(const ScanArgs& a, const WitnessBlock wb) {
+  DevResult* r = a.res + wb.mi;
+  const SyncTabs syt = sync_tabs_of(a, wb.mi);
+  const uint64_t s = __ldcg(&r->min_start);
+  if (s == ~0ull || __ldcg(&r->x_rank) == ~0ull) return;
+  const uint64_t e = __ldcg(&r->seg_end);
+  const uint64_t wcell = __ldcg(&r->cell);
   const uint32_t kb = a.thread_shift;
-  const unsigned long long xr = r->x_rank;
-  const uint32_t wb = syt.wp_bits;
-  const unsigned xw = (unsigned)(xr & ((1ull << wb) - 1ull));
-  const unsigned xk = (unsigned)(xr >> wb) & ((1u << kb) - 1u);
-  const unsigned xt = (unsigned)(xr >> (wb + kb)) & ((1u << a.thread_bits) - 1u);
-  const unsigned xp = (unsigned)(xr >> (wb + kb + a.thread_bits)) & ((1u << a.phase_bits) - 1u);
-  const unsigned b0 = (unsigned)(xr >> (wb + kb + a.thread_bits + a.phase_bits));   // x's block
+  const unsigned long long xr = __ldcg(&r->x_rank);
+  const uint32_t wpb = syt.wp_bits;
+  const unsigned xw = (unsigned)(xr & ((1ull << wpb) - 1ull));
+  const unsigned xk = (unsigned)(xr >> wpb) & ((1u << kb) - 1u);
+  const unsigned xt = (unsigned)(xr >> (wpb + kb)) & ((1u << a.thread_bits) - 1u);
+  const unsigned xp = (unsigned)(xr >> (wpb + kb + a.thread_bits)) & ((1u << a.phase_bits) - 1u);
+  const unsigned b0 = (unsigned)(xr >> (wpb + kb + a.thread_bits + a.phase_bits));   // x's block
   const unsigned xq = xp * syt.n_wp + xw;
   const unsigned xg = syt.on ? grid_q(a, syt, xq) : 0u;
   unsigned long long best = ~0ull;
-  for (uint64_t i = s + blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < e; i += (uint64_t)gridDim.x * blockDim.x) {
+  for (uint64_t i = s + wb.bi * (uint64_t)blockDim.x + threadIdx.x; i < e; i += (uint64_t)wb.nb * blockDim.x) {
     const uint64_t key = a.keys[i];
     if ((key >> a.cell_shift) != wcell) continue;   // the bucket path's range holds other cells too
     const Fields f = fields(a, key);
@@ -1331,7 +1344,7 @@ __global__ void __launch_bounds__(256) witness_y_kernel(ScanArgs a) {
     if (other_thread && kinds_conflict(xk, f.k) && concurrent) {
       const unsigned long long rank =
           ((((unsigned long long)f.b << (a.phase_bits + a.thread_bits + kb)) |
-            ((unsigned long long)yp << (a.thread_bits + kb)) | ((unsigned long long)f.t << kb) | f.k) << wb) | yw;
+            ((unsigned long long)yp << (a.thread_bits + kb)) | ((unsigned long long)f.t << kb) | f.k) << wpb) | yw;
       best = rank < best ? rank : best;
     }
   }
@@ -1343,32 +1356,75 @@ __global__ void __launch_bounds__(256) witness_y_kernel(ScanArgs a) {
   if ((threadIdx.x & 31) == 0 && best != ~0ull) atomicMin(&r->y_rank, best);
 }
 
+// the steps as kernels of their own: result blockIdx.y, the blocks of the x dimension
+__device__ __forceinline__ WitnessBlock grid_block() { return {blockIdx.y, blockIdx.x, gridDim.x}; }
+__global__ void __launch_bounds__(256) witness_cell_kernel(ScanArgs a) { witness_cell(a, grid_block()); }
+__global__ void __launch_bounds__(256) witness_group_kernel(ScanArgs a) { witness_group(a, grid_block()); }
+__global__ void __launch_bounds__(256) witness_x_kernel(ScanArgs a) { witness_x(a, grid_block()); }
+__global__ void __launch_bounds__(256) witness_y_kernel(ScanArgs a) { witness_y(a, grid_block()); }
+
+// The bucket of a result's smallest racy cell (bucket path), then the four steps,
+// in one launch: one cluster of C blocks per result.  A result without a racy
+// cell costs its launch alone.
+template <int C>
+__global__ void __launch_bounds__(512) witness_bucket_kernel(ScanArgs a, FinishArgs fa) {
+  const WitnessBlock wb{blockIdx.x / C, blockIdx.x % C, C};
+  DevResult* r = a.res + wb.mi;
+  const unsigned long long c = r->hash_cell;
+  if (c == ~0ull) return;   // (the whole cluster)
+  auto step = [] {
+    if constexpr (C > 1) cooperative_groups::this_cluster().sync();
+    else __syncthreads();
+  };
+  if (wb.bi == 0 && threadIdx.x == 0) bucket_of_racy_cell(fa, r, c);
+  step();
+  witness_cell(a, wb);
+  step();
+  witness_group(a, wb);
+  step();
+  witness_x(a, wb);
+  step();
+  witness_y(a, wb);
+}
+
+__device__ __forceinline__ void init_result(DevResult* r) {
+  r->oob_code = ~0ull;
+  r->instances = 0;
+  r->racy_cells = 0;
+  r->min_start = ~0ull;
+  r->seg_end = 0;
+  r->cell = 0;
+  r->x_rank = ~0ull;
+  r->y_rank = ~0ull;
+  r->minb = 0xffffffffu;
+  r->maxb = 0;
+  r->minWb = 0xffffffffu;
+  r->maxWb = 0;
+  r->anyW = 0;
+  r->minAb = r->minRb = 0xffffffffu;
+  r->maxAb = r->maxRb = 0;
+  r->anyA = r->anyR = 0;
+  r->err = 0;
+  r->n_keys = 0;
+  r->sorted_buf = 0;
+  r->hash_cell = ~0ull;
+  r->stop = 0;
+}
+
 __global__ void init_result_kernel(DevResult* res, uint32_t n) {
   const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) {
-    DevResult* r = res + i;
-    r->oob_code = ~0ull;
-    r->instances = 0;
-    r->racy_cells = 0;
-    r->min_start = ~0ull;
-    r->seg_end = 0;
-    r->cell = 0;
-    r->x_rank = ~0ull;
-    r->y_rank = ~0ull;
-    r->minb = 0xffffffffu;
-    r->maxb = 0;
-    r->minWb = 0xffffffffu;
-    r->maxWb = 0;
-    r->anyW = 0;
-    r->minAb = r->minRb = 0xffffffffu;
-    r->maxAb = r->maxRb = 0;
-    r->anyA = r->anyR = 0;
-    r->err = 0;
-    r->n_keys = 0;
-    r->sorted_buf = 0;
-    r->hash_cell = ~0ull;
-    r->stop = 0;
-  }
+  if (i < n) init_result(res + i);
+}
+
+// The start of a check: its result records (n of them, and one more), and what
+// has to be zero.
+__global__ void __launch_bounds__(256) init_check_kernel(DevResult* res, uint32_t n, DevResult* more, ulonglong2* zero,
+                                                         uint64_t n_zero, unsigned long long* queue) {
+  const uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
+  if (i < n) init_result(res + i);
+  if (i == 0 && more) init_result(more);
+  if (i == 0 && queue) *queue = 0;
+  for (uint64_t z = i; z < n_zero; z += (uint64_t)gridDim.x * blockDim.x) zero[z] = make_ulonglong2(0, 0);
 }
 
 }  // namespace
@@ -1376,6 +1432,23 @@ __global__ void init_result_kernel(DevResult* res, uint32_t n) {
 cudaError_t launch_init_result(DevResult* res, cudaStream_t st, uint32_t n) {
   if (n == 0) return cudaSuccess;
   init_result_kernel<<<(n + 127) / 128, 128, 0, st>>>(res, n);
+  return cudaGetLastError();
+}
+
+// One launch for the records and the cleared range; a range that takes more than
+// a few microseconds to clear goes to the memset.
+cudaError_t launch_init_check(DevResult* res, uint32_t n, DevResult* more, void* zero, size_t zero_bytes,
+                              unsigned long long* queue, cudaStream_t st) {
+  constexpr size_t kKernelClear = 4 << 20;
+  const bool big = zero_bytes > kKernelClear || ((reinterpret_cast<uintptr_t>(zero) | zero_bytes) & 15u) != 0u;
+  if (big) {
+    const cudaError_t e = cudaMemsetAsync(zero, 0, zero_bytes, st);
+    if (e != cudaSuccess) return e;
+  }
+  const uint64_t nz = big ? 0 : zero_bytes / 16;
+  const uint64_t work = std::max<uint64_t>(std::max<uint64_t>(n, 1), nz / 4);
+  init_check_kernel<<<(unsigned)((work + 255) / 256), 256, 0, st>>>(res, n, more, static_cast<ulonglong2*>(zero), nz,
+                                                                    queue);
   return cudaGetLastError();
 }
 
@@ -1416,6 +1489,7 @@ cudaError_t launch_scan(const ScanArgs& a, cudaStream_t st) {
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   }
+  if (a.by_cell) return cudaSuccess;   // (the first racy cell is known by value: launch_bucket_witness)
   const unsigned nr = a.n_models ? a.n_models : 1u;
   scan_finish_kernel<<<nr, 32, 0, st>>>(a);
   return cudaGetLastError();
@@ -1428,6 +1502,28 @@ cudaError_t launch_witness(const ScanArgs& a, cudaStream_t st) {
   witness_x_kernel<<<g, 256, 0, st>>>(a);
   witness_y_kernel<<<g, 256, 0, st>>>(a);
   return cudaGetLastError();
+}
+
+cudaError_t launch_bucket_witness(const ScanArgs& a, const FinishArgs& fa, cudaStream_t st) {
+  if (a.n_models) {
+    witness_bucket_kernel<1><<<a.n_models, 512, 0, st>>>(a, fa);
+    return cudaGetLastError();
+  }
+  if (a.n > kWitnessClusterKeys) {
+    const cudaError_t e = launch_bucket_finish(fa, st);
+    return e == cudaSuccess ? launch_witness(a, st) : e;
+  }
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(kWitnessCluster);
+  cfg.blockDim = dim3(512);
+  cfg.stream = st;
+  cudaLaunchAttribute at;
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.x = kWitnessCluster;
+  at.val.clusterDim.y = at.val.clusterDim.z = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, witness_bucket_kernel<kWitnessCluster>, a, fa);
 }
 
 uint64_t scan_long_capacity(uint64_t n, uint32_t n_warps) {
