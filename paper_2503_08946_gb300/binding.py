@@ -631,12 +631,7 @@ class RcServer:
             pass
 
 
-def rc_report_array(ticket, wait: bool = True):
-    """The results of a ticket as one numpy record array, one record per
-    model with the fields of ``rc_result`` (``x``/``y`` are records of the
-    fields of ``rc_inst``).  No Python object is made per result: a batch of
-    10,000 models decodes in about a millisecond instead of tens."""
-    import numpy as np
+def _report(ticket, wait: bool):
     t, n = ticket
     out = (rc_result * max(1, n))()
     st = load().rc_report(c_void_p(t), out, 1 if wait else 0)
@@ -644,7 +639,23 @@ def rc_report_array(ticket, wait: bool = True):
         raise NotReady()
     if st != RC_OK:
         raise RcError(st, "rc_report")
-    return np.ctypeslib.as_array(out)[:n]
+    return out, n
+
+
+_RESULT_DTYPE = None   # numpy's view of rc_result; deriving it takes longer than a small check
+
+
+def rc_report_array(ticket, wait: bool = True):
+    """The results of a ticket as one numpy record array, one record per
+    model with the fields of ``rc_result`` (``x``/``y`` are records of the
+    fields of ``rc_inst``).  No Python object is made per result: a batch of
+    10,000 models decodes in about a millisecond instead of tens."""
+    global _RESULT_DTYPE
+    import numpy as np
+    out, n = _report(ticket, wait)
+    if _RESULT_DTYPE is None:
+        _RESULT_DTYPE = np.ctypeslib.as_array(out).dtype
+    return np.frombuffer(out, dtype=_RESULT_DTYPE)[:n]
 
 
 def results_of(arr) -> List[Result]:
@@ -658,7 +669,12 @@ def results_of(arr) -> List[Result]:
 
 
 def rc_report(ticket, wait: bool = True) -> List[Result]:
-    return results_of(rc_report_array(ticket, wait))
+    if ticket[1] > 4:
+        return results_of(rc_report_array(ticket, wait))
+    # few results: straight from the structure (a numpy array of one record costs
+    # five times the decoding)
+    out, n = _report(ticket, wait)
+    return [_result(out[i]) for i in range(n)]
 
 
 def rc_ticket_stage_times(ticket) -> dict:
