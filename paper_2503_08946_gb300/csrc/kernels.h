@@ -63,13 +63,19 @@ struct BatchArgs {
   uint32_t n_models;
   uint64_t n_units;
   unsigned long long* queue;     // starts at 0
+  uint32_t grab;                 // units a block takes at once (set by the launcher)
   uint64_t* keys;                // batch key buffer
   DevResult* res;                // one per model
   uint32_t cell_shift, phase_shift, block_shift;   // batch key layout
   uint32_t thread_shift;                           // = the batch's kind field bits
 };
-// loop_free: every statement of the pack's models has no loops
-cudaError_t launch_batch_expand(const BatchArgs& a, bool loop_free, cudaStream_t st);
+// loop_free: every statement of the pack's models has no loops.  flat: model
+// threads per lane of the expansion for loop-free models with one-dimensional
+// grids and blocks (a unit is then flat * kExpandThreadsHost threads), 0 = the
+// general kernels; max_terms: most terms of a statement of the pack.
+constexpr uint32_t kBatchFlatThreads = 4;
+cudaError_t launch_batch_expand(const BatchArgs& a, bool loop_free, uint32_t flat, uint32_t max_terms,
+                                cudaStream_t st);
 cudaError_t launch_batch_errors(const DevResult* pack, DevResult* res, uint32_t n, cudaStream_t st);
 
 // hash.cu

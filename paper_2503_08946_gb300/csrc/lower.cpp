@@ -650,6 +650,7 @@ rc_status lower_model(const rc_model_desc* d, Model* m, std::vector<int32_t>* ge
     D.n_key = n_key;
     D.term0 = (int32_t)terms.size();
     D.n_terms = (int32_t)b.terms.size();
+    if (b.terms.size() > m->max_terms) m->max_terms = (uint32_t)b.terms.size();
     for (size_t q = 0; q < b.terms.size(); ++q) {
       Term t;
       t.row = (int32_t)rows.size();

@@ -1092,12 +1092,17 @@ struct BatchPack {
   uint32_t tb = 0, bb = 0, pb = 0, cell_bits = 0;
   uint32_t kb = 1;                     // kind field bits (2 if some model has atomics)
   bool loop_free = true;               // every model of the pack is loop-free
+  bool one_dim = true;                 // ... and has one-dimensional grids and blocks
+  uint32_t max_terms = 0;              // most terms of a statement of its models
+  uint32_t flat = 0;                   // model threads per lane of the flat expansion, 0 = general kernels
   bool sy = false;                     // some model has warp or grid barriers
   bool mg = false;                     // its models have more than one grid interval (per-block witness groups)
   const uint32_t* grid_of = nullptr;   // phase-order scan with warp / grid barriers: its model's interval table
   uint64_t total_cells = 0, n_keys = 0, n_units = 0;
   rc::WorkspacePlan p;                 // sort / scan sections (offsets into the shared pack region)
 };
+
+constexpr uint64_t kBatchFlatMinUnits = 152 * 8;
 
 struct BatchLayout {
   std::vector<BatchPack> packs;
@@ -1106,8 +1111,14 @@ struct BatchLayout {
   size_t total = 0;
 };
 
-uint32_t chunks_of(const rc::Model& m) {
-  return (uint32_t)((m.host.n_threads + rc::kExpandThreadsHost - 1) / rc::kExpandThreadsHost);
+// expansion units of a model in a pack with `flat` model threads per lane
+uint32_t chunks_of(const rc::Model& m, uint32_t flat) {
+  const uint64_t t = (uint64_t)rc::kExpandThreadsHost * (flat ? flat : 1u);
+  return (uint32_t)((m.host.n_threads + t - 1) / t);
+}
+bool one_dim(const rc::Model& m) {
+  const rc::DevModel& h = m.host;
+  return h.block[1] == 1 && h.block[2] == 1 && h.grid[1] == 1 && h.grid[2] == 1 && h.n_threads < (1ull << 32);
 }
 
 rc_status plan_batch(rc_model* const* models, size_t n, const rc_check_opts* opts, BatchLayout* L) {
@@ -1135,9 +1146,10 @@ rc_status plan_batch(rc_model* const* models, size_t n, const rc_check_opts* opt
       if (cells >= cur.total_cells && table_ok && mg_ok && kb + tb + bb + pb + cb <= (uint32_t)rc::kKeyBits) {
         cur.tb = tb; cur.bb = bb; cur.pb = pb; cur.kb = kb; cur.total_cells = cells; cur.cell_bits = cb;
         cur.loop_free = cur.loop_free && m.loop_free;
+        cur.one_dim = cur.one_dim && one_dim(m);
+        cur.max_terms = std::max(cur.max_terms, m.max_terms);
         cur.sy = sy;
         cur.n_keys += m.key_slots;
-        cur.n_units += chunks_of(m);
         cur.i1 = i + 1;
         continue;
       }
@@ -1148,6 +1160,8 @@ rc_status plan_batch(rc_model* const* models, size_t n, const rc_check_opts* opt
     cur.i1 = i + 1;
     cur.tb = h.thread_bits; cur.bb = h.block_bits; cur.pb = h.phase_bits; cur.kb = h.thread_shift;
     cur.loop_free = m.loop_free;
+    cur.one_dim = one_dim(m);
+    cur.max_terms = m.max_terms;
     cur.sy = m.sync_scopes;
     cur.mg = m.multi_grid;
     // (a model scanned in phase order with warp or grid barriers holds its pack alone)
@@ -1157,10 +1171,24 @@ rc_status plan_batch(rc_model* const* models, size_t n, const rc_check_opts* opt
     cur.total_cells = m.total_cells;
     cur.cell_bits = rc::bit_length(m.total_cells);
     cur.n_keys = m.key_slots;
-    cur.n_units = chunks_of(m);
     open = true;
   }
   if (open) L->packs.push_back(cur);
+  for (BatchPack& k : L->packs) {
+    // the flat expansion where it applies, with several model threads per lane
+    // where that leaves enough units for the GPU
+    auto units = [&](uint32_t flat) {
+      uint64_t u = 0;
+      for (size_t i = k.i0; i < k.i1; ++i) u += chunks_of(models[i]->m, flat);
+      return u;
+    };
+    k.flat = k.loop_free && k.one_dim ? rc::kBatchFlatThreads : 0u;
+    k.n_units = units(k.flat);
+    if (k.flat > 1 && k.n_units < kBatchFlatMinUnits) {
+      k.flat = 1;
+      k.n_units = units(1);
+    }
+  }
   // per-model records and tables, then one pack region sized for the largest pack
   size_t off = 0;
   L->res_off = off;
@@ -1259,7 +1287,7 @@ void fill_batch_tables(rc_model* const* models, const BatchLayout& L, void* uplo
       b.unit_base = unit_base;
       b.n_threads = h.n_threads;
       b.n_stmts = h.n_stmts;
-      b.n_chunks = chunks_of(m);
+      b.n_chunks = chunks_of(m, k.flat);
       b.cell_shift = h.cell_shift;
       b.phase_shift = h.phase_shift;
       b.block_shift = h.block_shift;
@@ -1313,7 +1341,7 @@ rc_status enqueue_batch_device(const BatchLayout& L, size_t n, const rc_check_op
     ba.phase_shift = k.kb + k.tb + k.bb;
     ba.block_shift = k.kb + k.tb;
     ba.cell_shift = ba.phase_shift + k.pb;
-    s = cuda_status(rc::launch_batch_expand(ba, k.loop_free, st));
+    s = cuda_status(rc::launch_batch_expand(ba, k.loop_free, k.flat, k.max_terms, st));
     if (s != RC_OK) break;
     int sorted = 0;
     if (!p.bucket.on) {
