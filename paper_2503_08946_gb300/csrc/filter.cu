@@ -39,7 +39,9 @@
 // 49 M keys with hot cells 0.26 ms against 1.63 + 0.22 ms.  Blocks of 256 threads
 // with 20 keys each in registers, 4 per SM, were the fastest split without spills
 // (512 threads, 2 per SM: 1.95 ms; 384 threads with 16 keys, 3 per SM: 1.51 ms):
-// the barriers between the steps stall fewer warps.
+// the barriers between the steps stall fewer warps.  The hashed table (HT) takes
+// 3 blocks per SM; on 2,000 small models in one batch (34 cell bits, 18 million
+// kept keys) the check takes 1.99 ms with it, 2.62 ms with the local sort and scan.
 #include <cuda_runtime.h>
 
 #include "fold.cuh"
@@ -56,6 +58,11 @@ constexpr int kFltKPT = 20;                        // keys per thread held in re
 constexpr int kFltStreamKPT = 12;                  // keys per thread and step of a larger bucket
 constexpr unsigned kFltCap = kFltThreads * kFltKPT;
 static_assert((1 << kFilterMaxSlotBits) / 32 <= kFltThreads, "a word of a bit mask per thread");
+static_assert(kFltCap < (1 << kFilterMaxSlotBits), "a bucket in registers leaves free slots in a hashed table");
+constexpr unsigned kNoTag = 0xffffffffu;           // (tags have at most 31 bits)
+constexpr unsigned kTagMul = 0x9E3779B1u;          // home slot of a tag (Fibonacci hashing: its low bits alone
+                                                   // are those of the cell's low bits, equal for equal strides)
+constexpr unsigned kPartMul = 0x85EBCA77u;         // part of a tag (odd: 32 part bits tell all tags apart)
 
 // inverse of the odd hash multiplier modulo 2^64 (Newton's iteration: each step
 // doubles the number of correct low bits)
@@ -66,16 +73,19 @@ constexpr uint64_t hash_inverse() {
 }
 static_assert(hash_inverse() * kCellHashMul == 1ull, "inverse of the cell hash multiplier");
 
-// words of the representative table: a slot per cell, and room for at least
-// 256 candidate cells of 16 intervals each
+// Slots of a table.  Direct (r <= kFilterMaxSlotBits): the slot is the cell's r
+// hash bits, and the table has room for at least 256 candidate cells of 16
+// intervals each.  Hashed (HT, larger r): 2^kFilterMaxSlotBits slots with a tag.
 __host__ __device__ __forceinline__ unsigned table_words(uint32_t r) {
-  return r < 12 ? 4096u : (1u << r);
+  return r < 12 ? 4096u : r > kFilterMaxSlotBits ? 1u << kFilterMaxSlotBits : 1u << r;
 }
-__host__ __device__ __forceinline__ unsigned mask_words(uint32_t r) { return r < 5 ? 1u : (1u << (r - 5)); }
-// (four words behind the table: the slot of padding keys)
+__host__ __device__ __forceinline__ unsigned mask_words(uint32_t r) {
+  return r < 5 ? 1u : r > kFilterMaxSlotBits ? 1u << (kFilterMaxSlotBits - 5) : 1u << (r - 5);
+}
+// (four words behind the table: the slot of padding keys and of cells without a write)
 size_t filter_smem(uint32_t r, bool at) {
-  return ((size_t)table_words(r) + 4 + (at ? 10 : 5) * (size_t)mask_words(r) + 1 + (at ? 3 * table_words(r) / 32 : 0)) *
-         sizeof(unsigned);
+  const size_t tw = table_words(r), mw = mask_words(r);
+  return (tw + 4 + (r > kFilterMaxSlotBits ? tw : 0) + (at ? 10 : 5) * mw + 1 + (at ? 3 * tw / 32 : 0)) * sizeof(unsigned);
 }
 
 // One block per bucket.  A bucket of at most kFltCap keys is held in registers
@@ -83,11 +93,18 @@ size_t filter_smem(uint32_t r, bool at) {
 // a thread past the bucket's end repeat its first key (the same instance, which
 // changes nothing), so no step tests for them; PAD: the bucket holds padding
 // keys (the unpartitioned single bucket), held as reads of the word behind the table.
-template <bool PAD, bool REGS, bool AT>
+// HT: the cell space is too sparse for a slot per cell.  The written cells take
+// slots of an open-addressed table (the cell's r hash bits are its tag), and
+// every key looks its cell up: not found, it has no write and cannot race.  A
+// bucket in registers has fewer keys than the table has slots.  A larger one may
+// hold more written cells: where the table runs out, its cells are taken in
+// halves, quarters and so on by another hash of the tag.
+template <bool PAD, bool REGS, bool AT, bool HT>
 __device__ __forceinline__ void filter_bucket(const FilterArgs& a, const uint64_t* src, uint64_t len) {
   extern __shared__ __align__(16) unsigned s_tab[];
   const unsigned tw = table_words(a.r), mw = mask_words(a.r);
-  unsigned* s_two = s_tab + tw + 4;     // cells with two threads of a block, a bit per slot
+  unsigned* s_tag = s_tab + tw + 4;     // (HT) the cell of every slot
+  unsigned* s_two = s_tag + (HT ? tw : 0u);   // cells with two threads of a block, a bit per slot
   unsigned* s_wi = s_two + mw;          // cells with writes in two intervals, then the candidate cells
   unsigned* s_racy = s_wi + mw;         // racy cells
   unsigned* s_hot = s_racy + mw;        // racy candidate cells, a bit per candidate
@@ -111,18 +128,31 @@ __device__ __forceinline__ void filter_bucket(const FilterArgs& a, const uint64_
                  m_b = (unsigned)(((1ull << bb) - 1ull) << (kb + tb)),
                  m_p = (unsigned)(((1ull << pb) - 1ull) << (kb + tb + bb));
   const uint32_t cs = a.s.cell_shift;
-  const unsigned smask = (1u << a.r) - 1u;
+  const unsigned smask = (1u << a.r) - 1u;   // (r <= 31)
+  uint32_t part_bits = 0, part = 0;          // (HT, not REGS) the part of the bucket's cells in hand
   const unsigned lmask = cs < 32 ? (1u << cs) - 1u : ~0u;
-  // low word and slot of a key (the low r bits of the hash depend on the low bits
-  // of the cell alone)
+  // low word and slot (HT: tag) of a key (the low r bits of the hash depend on the
+  // low bits of the cell alone)
   auto unpack = [&](uint64_t k, unsigned& kl, unsigned& sl) {
     kl = (uint32_t)k & lmask;
     sl = (__funnelshift_rc((uint32_t)k, (uint32_t)(k >> 32), cs) * (uint32_t)kCellHashMul) & smask;
     if (PAD && k == kSentinel) {
-      sl = tw;
+      sl = HT ? kNoTag : tw;
       kl = 0;
     }
   };
+  // the slot of a cell, or tw if it has none
+  constexpr unsigned kProbes = REGS ? (1u << kFilterMaxSlotBits) : 512u;
+  auto find = [&](unsigned tag) -> unsigned {
+    unsigned i = (tag * kTagMul) >> (32 - kFilterMaxSlotBits);
+    for (unsigned n = 0; n < kProbes; ++n, i = (i + 1u) & (tw - 1u)) {
+      const unsigned t = s_tag[i];
+      if (t == tag) return i;
+      if (t == kNoTag) break;
+    }
+    return tw;
+  };
+  auto in_part = [&](unsigned tag) { return part_bits == 0u || (tag * kPartMul) >> (32u - part_bits) == part; };
   unsigned rl[kFltKPT], rs[kFltKPT];   // (REGS) the bucket
   const int nq = REGS ? (int)((len + kFltThreads - 1) / kFltThreads) : 0;
   if constexpr (REGS) {
@@ -141,6 +171,7 @@ __device__ __forceinline__ void filter_bucket(const FilterArgs& a, const uint64_
       unpack(k[q], rl[q], rs[q]);
     }
   }
+  bool resolve = false;   // (HT, not REGS) whether the written cells have their slots
   // f(low word, slot) for the keys of the bucket
   auto each = [&](auto&& f) {
     if constexpr (REGS) {
@@ -163,6 +194,10 @@ __device__ __forceinline__ void filter_bucket(const FilterArgs& a, const uint64_
         for (int u = 0; u < kFltStreamKPT; ++u) {
           unsigned kl, sl;
           unpack(k[u], kl, sl);
+          if constexpr (HT) {
+            if (!in_part(sl)) continue;
+            if (resolve) sl = find(sl);
+          }
           f(kl, sl);
         }
       }
@@ -176,10 +211,39 @@ __device__ __forceinline__ void filter_bucket(const FilterArgs& a, const uint64_
     const unsigned bit = 1u << (i & 31u);
     if (!(bits[i >> 5] & bit)) atomicOr(&bits[i >> 5], bit);
   };
+  // one test of the bucket's cells (HT: of those in hand); false: the table ran out
+  auto test = [&]() -> bool {
+  resolve = false;
   // (the slots rounded up to whole 16-byte stores lie inside the table)
-  clear_table(PAD ? tw + 4u : ((1u << a.r) + 3u) & ~3u);
+  clear_table(PAD || HT ? tw + 4u : ((1u << a.r) + 3u) & ~3u);
+  if constexpr (HT)
+    for (unsigned i = 4 * tid; i < tw; i += 4 * kFltThreads)
+      *reinterpret_cast<uint4*>(s_tag + i) = make_uint4(kNoTag, kNoTag, kNoTag, kNoTag);
   for (unsigned i = tid; i < (AT ? 10 : 4) * mw + 1; i += kFltThreads) s_two[i] = 0;
   __syncthreads();
+  if constexpr (HT) {
+    // 0. a slot for every written cell, then every key's slot
+    bool full = false;
+    each([&](unsigned k, unsigned tag) {
+      if ((k & kmask) == 0u) return;
+      unsigned i = (tag * kTagMul) >> (32 - kFilterMaxSlotBits), n = 0;
+      for (; n < kProbes; ++n, i = (i + 1u) & (tw - 1u)) {
+        unsigned t = s_tag[i];
+        if (t == kNoTag) t = atomicCAS(&s_tag[i], kNoTag, tag);
+        if (t == kNoTag || t == tag) break;
+      }
+      full = full || n == kProbes;
+    });
+    if (__syncthreads_or(full)) return false;
+    resolve = true;
+    if constexpr (REGS) {
+#pragma unroll
+      for (int q = 0; q < kFltKPT; ++q) {
+        if (q >= nq) break;
+        rs[q] = find(rs[q]);
+      }
+    }
+  }
   // 1. the representative of every written cell (its low word is not 0)
   bool any = false;
   each([&](unsigned k, unsigned s) {
@@ -188,7 +252,7 @@ __device__ __forceinline__ void filter_bucket(const FilterArgs& a, const uint64_
       any = true;
     }
   });
-  if (!__syncthreads_or(any)) return;   // no write: nothing can race
+  if (!__syncthreads_or(any)) return true;   // no write: nothing can race
   // 2. every key against its cell's representative
   any = false;
   each([&](unsigned k, unsigned s) {
@@ -214,7 +278,7 @@ __device__ __forceinline__ void filter_bucket(const FilterArgs& a, const uint64_
       if ((k & 1u) && (d & m_p)) mark(s_wi, s);
     }
   });
-  if (!__syncthreads_or(any)) return;   // every written cell has one thread and interval
+  if (!__syncthreads_or(any)) return true;   // every written cell has one thread and interval
   // 3. the candidate cells numbered in slot order; at most one word of a bit
   // mask per thread
   unsigned cand = 0;
@@ -249,7 +313,7 @@ __device__ __forceinline__ void filter_bucket(const FilterArgs& a, const uint64_
     __syncthreads();
     // the entry (candidate << pb | interval) of a key, ~0 if its cell is no candidate
     auto entry = [&](unsigned k, unsigned s) -> unsigned {
-      if (PAD && s == tw) return ~0u;
+      if ((PAD || HT) && s == tw) return ~0u;
       const unsigned m = s_wi[s >> 5];
       if (!((m >> (s & 31u)) & 1u)) return ~0u;
       return ((s_rank[s >> 5] + __popc(m & ((1u << (s & 31u)) - 1u))) << pb) | (unsigned)((uint64_t)k >> (kb + bb + tb));
@@ -291,7 +355,7 @@ __device__ __forceinline__ void filter_bucket(const FilterArgs& a, const uint64_
     }
   }
   // the racy cells: counted, and the smallest by value kept.  Slot s of bucket b
-  // has hash (part | b | s), whose cell is hash * inverse mod 2^(cell bits).
+  // (HT: its tag) has hash (part | b | s), whose cell is hash * inverse mod 2^(cell bits).
   const uint64_t inv = hash_inverse();
   unsigned count = 0;
   unsigned long long first = ~0ull;
@@ -308,7 +372,7 @@ __device__ __forceinline__ void filter_bucket(const FilterArgs& a, const uint64_
     while (m) {
       const unsigned slot = 32u * tid + (unsigned)__ffs(m) - 1u;
       m &= m - 1u;
-      const uint64_t h = a.part_hash | ((uint64_t)blockIdx.x << a.r) | slot;
+      const uint64_t h = a.part_hash | ((uint64_t)blockIdx.x << a.r) | (HT ? s_tag[slot] : slot);
       const uint64_t cell = (h * inv) & a.hmask;
       if (a.s.n_models) {
         DevResult* r = result_of(a.s, cell);
@@ -319,42 +383,67 @@ __device__ __forceinline__ void filter_bucket(const FilterArgs& a, const uint64_
       }
     }
   }
-  if (a.s.n_models) return;
+  if (a.s.n_models) return true;
   count = __reduce_add_sync(FULL, count);
-  if (count == 0) return;
+  if (count == 0) return true;
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) first = min(first, __shfl_xor_sync(FULL, first, o));
   if (lane == 0) {
     atomicAdd(&a.s.res->racy_cells, (unsigned long long)count);
     atomicMin(&a.s.res->hash_cell, first);
   }
+  return true;
+  };
+  if constexpr (REGS || !HT) {
+    test();
+  } else {
+    // the parts (part_bits, part) in order; one that is too large is halved
+    do {
+      if (!test()) {
+        ++part_bits;
+        part *= 2u;
+      } else {
+        ++part;
+        while (part_bits != 0u && (part & 1u) == 0u) {
+          part >>= 1;
+          --part_bits;
+        }
+      }
+      __syncthreads();
+    } while (part_bits != 0u || part == 0u);
+  }
 }
 
-template <bool PAD, bool AT>
-__global__ void __launch_bounds__(kFltThreads, kFltBlocks) bucket_filter_kernel(FilterArgs a) {
+template <bool PAD, bool AT, bool HT>
+__global__ void __launch_bounds__(kFltThreads, HT ? 3 : kFltBlocks) bucket_filter_kernel(FilterArgs a) {
   const uint64_t lo = a.boff[blockIdx.x], hi = a.boff[blockIdx.x + 1];
   if (hi < lo + 2) return;              // a race needs two keys
-  if (hi - lo <= (uint64_t)kFltCap) filter_bucket<PAD, true, AT>(a, a.keys_in + lo, hi - lo);
-  else filter_bucket<PAD, false, AT>(a, a.keys_in + lo, hi - lo);
+  if (hi - lo <= (uint64_t)kFltCap) filter_bucket<PAD, true, AT, HT>(a, a.keys_in + lo, hi - lo);
+  else filter_bucket<PAD, false, AT, HT>(a, a.keys_in + lo, hi - lo);
 }
 
-template <bool PAD, bool AT>
+template <bool PAD, bool AT, bool HT>
 cudaError_t launch_filter(const FilterArgs& a, uint32_t D, cudaStream_t st) {
-  const cudaError_t e = ensure_kernel_smem(reinterpret_cast<const void*>(bucket_filter_kernel<PAD, AT>),
-                                           filter_smem(kFilterMaxSlotBits, AT));
+  const cudaError_t e = ensure_kernel_smem(reinterpret_cast<const void*>(bucket_filter_kernel<PAD, AT, HT>),
+                                           filter_smem(HT ? 31 : kFilterMaxSlotBits, AT));
   if (e != cudaSuccess) return e;
-  bucket_filter_kernel<PAD, AT><<<1u << D, kFltThreads, filter_smem(a.r, AT), st>>>(a);
+  bucket_filter_kernel<PAD, AT, HT><<<1u << D, kFltThreads, filter_smem(a.r, AT), st>>>(a);
   return cudaGetLastError();
+}
+template <bool PAD>
+cudaError_t launch_filter(const FilterArgs& a, uint32_t D, cudaStream_t st) {
+  const bool at = a.s.thread_shift == 2;
+  if (a.r > kFilterMaxSlotBits)
+    return at ? launch_filter<PAD, true, true>(a, D, st) : launch_filter<PAD, false, true>(a, D, st);
+  return at ? launch_filter<PAD, true, false>(a, D, st) : launch_filter<PAD, false, false>(a, D, st);
 }
 
 }  // namespace
 
 cudaError_t launch_bucket_filter(const FilterArgs& a, uint32_t D, cudaStream_t st) {
-  if (a.r > kFilterMaxSlotBits || a.s.cell_shift > kFilterMaxLowBits) return cudaErrorInvalidValue;
+  if (a.r > kFilterMaxTagBits || a.s.cell_shift > kFilterMaxLowBits) return cudaErrorInvalidValue;
   // an unpartitioned bucket holds padding keys, which take the word behind the table
-  const bool at = a.s.thread_shift == 2;
-  if (D == 0) return at ? launch_filter<true, true>(a, D, st) : launch_filter<true, false>(a, D, st);
-  return at ? launch_filter<false, true>(a, D, st) : launch_filter<false, false>(a, D, st);
+  return D == 0 ? launch_filter<true>(a, D, st) : launch_filter<false>(a, D, st);
 }
 
 }  // namespace rc

@@ -245,15 +245,14 @@ struct LocalSortArgs {
 };
 cudaError_t launch_bucket_local_sort(const LocalSortArgs& a, cudaStream_t st);
 // filter.cu: the cell test of the bucket path without a sort, for models without
-// atomics and without warp or grid barriers whose cells have a table slot each
-// in every bucket (BucketPlan.filter): counts the racy cells of every bucket
+// warp or grid barriers (BucketPlan.filter): counts the racy cells of every bucket
 // [boff[b], boff[b+1]) of keys_in and keeps the smallest by value
 // (DevResult.racy_cells, hash_cell).
 struct FilterArgs {
   ScanArgs s;                       // key layout, results, models of a batch (keys, n and the scan's lists unused)
   const uint64_t* keys_in;
   const unsigned long long* boff;
-  uint32_t r;                       // hash bits below the bucket bits = slot bits (at most kFilterMaxSlotBits)
+  uint32_t r;                       // hash bits below the bucket bits = slot bits (tag bits above kFilterMaxSlotBits)
   uint64_t hmask;                   // 2^(cell bits) - 1 of the whole hash
   uint64_t part_hash;               // a hash part's top bits of the hash, 0 for a whole check
 };

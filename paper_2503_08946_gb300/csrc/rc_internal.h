@@ -347,10 +347,11 @@ constexpr int kPartTileHost = kSortThreadsHost * 16;    // keys per tile of the 
 
 // The cell test in shared memory (filter.cu).  The target keeps a bucket's keys
 // inside its block's registers (5,120) with room for the spread; 6,000 and 9,000
-// keys with larger blocks measured slower.  Fewer keys per bucket than
-// kFilterMinKeys would clear and scan a mostly empty table: the local sort's
-// buckets then cost less.
+// keys with larger blocks measured slower.  A slot per cell needs cell bits -
+// kFilterMaxSlotBits bucket bits; where that makes buckets of fewer than
+// kFilterMinKeys keys (mostly empty tables), the tables are hashed.
 constexpr uint32_t kFilterMaxSlotBits = 13;         // table slots of a bucket: 32 KB of 4-byte words
+constexpr uint32_t kFilterMaxTagBits = 31;          // hash bits below the bucket bits, with a hashed table
 constexpr uint32_t kFilterMaxLowBits = 32;          // (interval, block, thread, kind) bits: a table word
 constexpr uint64_t kFilterTarget = 4600;            // planned mean keys per bucket (at most)
 constexpr uint64_t kFilterMinKeys = 512;            // ... and at least, where the cell bits ask for more buckets

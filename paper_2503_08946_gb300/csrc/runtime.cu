@@ -229,21 +229,18 @@ static bool filter_allowed(bool sync_scopes, uint32_t cell_shift) {
 
 // n key slots, of which about n_expect are kept (a hash-partitioned check keeps
 // its share): the bucket count is chosen for n_expect, the tile bounds for n
-// Bucket bits of the table test, or ~0 where it does not pay: enough buckets
-// that every cell has its own slot and a bucket's keys fit the registers.
+// Bucket bits of the table test, or ~0 where it does not apply.
 static uint32_t filter_bucket_bits(uint64_t n_expect, uint32_t cb) {
   uint32_t D = 0;
   while (D < cb && D < kBucketMaxBits && (n_expect >> D) > kFilterTarget) ++D;
-  const uint32_t need = cb > kFilterMaxSlotBits ? cb - kFilterMaxSlotBits : 0u;
-  if (need > kBucketMaxBits) return ~0u;
+  if (D == kBucketMaxBits && (n_expect >> D) > kFilterTarget) return ~0u;
+  const uint32_t need = cb > kFilterMaxSlotBits ? cb - kFilterMaxSlotBits : 0u;   // for a slot per cell
   // one partition pass where its buckets stay small enough to be read again from L2
   const uint32_t one = kBucketMaxDigitBits;
-  if (D > one && cb <= one + kFilterMaxSlotBits && (n_expect >> one) <= kFilterOnePassKeys) return one;
-  if (need > D) {
-    if ((n_expect >> need) < kFilterMinKeys) return ~0u;   // a sparse cell space: mostly empty tables
-    D = need;
-  }
-  return D;
+  if (D > one && need <= one && (n_expect >> one) <= kFilterOnePassKeys) return one;
+  if (need <= D) return D;
+  if (need <= kBucketMaxBits && (n_expect >> need) >= kFilterMinKeys) return need;
+  return cb - D <= kFilterMaxTagBits ? D : ~0u;   // a sparse cell space: hashed tables
 }
 
 bool plan_buckets(uint64_t n, uint64_t n_expect, uint32_t cb, uint32_t phase_bits, bool filter_ok, size_t off,

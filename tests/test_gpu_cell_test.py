@@ -8,7 +8,7 @@ import pytest
 import oracle
 import workloads as w
 from workloads.rng import SplitMix64
-from workloads.spec import A, Access, Array, GLOBAL, Loop, Model, R, SHARED, Stmt, W, bid, const, it, tid
+from workloads.spec import A, Access, Array, GLOBAL, Loop, Model, R, SHARED, Stmt, W, bid, const, it, load, tid
 
 pytestmark = pytest.mark.gpu
 
@@ -135,3 +135,56 @@ def test_many_intervals(rc, phases):
     check(rc, m)
     check(rc, atomic_mix(7, 300, 256, 50, phases, SHARED))
     check(rc, atomic_mix(8, 300, 256, 3000, phases, GLOBAL))
+
+
+# ---- hashed tables (cell spaces too sparse for a slot per cell) ----
+
+@pytest.mark.parametrize("row_bits", [8, 16, 20, 24])
+@pytest.mark.parametrize("blocks", [1, 9, 64])
+def test_sparse_rows(rc, row_bits, blocks):
+    check(rc, w.random_affine(11 + row_bits, n_blocks=blocks, block=64, n_stmts=20, plant=True,
+                              row_global=1 << row_bits))
+
+
+def same_bucket(n, atomic=False, cb=24):
+    """n cells that share the top hash bits (hash values 0 .. n - 1), so that they
+    lie in one bucket: more written cells than its table has slots.  Thread t
+    writes cell t; every third cell is read by the next thread, every fifth in
+    the same interval."""
+    inv = pow(0x9E3779B97F4A7C15, -1, 1 << 64)
+    cells = [(h * inv) % (1 << cb) for h in range(n)]
+    cells = [c if c < (1 << cb) - 1 else 0 for c in cells]
+    a = Array("a", GLOBAL, ((1 << cb) - 1,))
+    block = 250
+    g = bid.x * block + tid.x
+    kind = A if atomic else W
+    stmts = [Stmt([Access(0, kind, (load(0, g),))], phase=const(0)),
+             Stmt([Access(0, R, (load(0, (g + 1) % n),))], phase=const(1), guards=[const(0) - g % 3]),
+             Stmt([Access(0, R, (load(0, (g + 7) % n),))], phase=const(0), guards=[const(0) - g % 5, const(100) - bid.x])]
+    return Model((n // block, 1, 1), (block, 1, 1), [a], stmts, n_phases=2, tables=[cells], name=f"same_bucket{n}")
+
+
+@pytest.mark.parametrize("atomic", [False, True])
+@pytest.mark.parametrize("n", [250, 1500, 8000, 20000, 40000])
+def test_more_written_cells_than_slots(rc, n, atomic):
+    check(rc, same_bucket(n, atomic))
+
+
+@pytest.mark.parametrize("seed", range(6))
+def test_sparse_atomics_and_batches(rc, seed):
+    rng = SplitMix64(seed)
+    big = Array("a", GLOBAL, (5000, 1 << 17))
+    ms = []
+    for k in range(7):
+        i = (rng.uniform_int(1, 4) * tid.x + rng.uniform_int(0, 9) * bid.x) % 5000
+        st = [Stmt([Access(0, (R, W, A)[rng.below(3)], (i + const(j % 2), const((1 << 16) + 3 * j)))],
+                   phase=const(rng.below(3))) for j in range(4)]
+        ms.append(Model((1 + rng.below(40), 1, 1), (32 * (1 + rng.below(4)), 1, 1), [big], st, n_phases=3, name=f"sp{k}"))
+    exp = [oracle.check(m) for m in ms]
+    for m, e in zip(ms, exp):
+        got = rc.check(m)
+        assert (got.status, got.racy_cells, got.witness) == (e.status, e.racy_cells, e.witness), m.name
+    h = [rc.rc_model_create(m) for m in ms]
+    got = rc.rc_report(rc.rc_check_batch(h, None, rc.workspace(rc.rc_batch_workspace_size(h, None))))
+    assert [(g.status, g.instances, g.racy_cells, g.witness) for g in got] == \
+        [(e.status, e.instances, e.racy_cells, e.witness) for e in exp]
