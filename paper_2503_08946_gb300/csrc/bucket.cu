@@ -158,7 +158,7 @@ __global__ void __launch_bounds__(1024) bucket_scan_a_kernel(BucketArgs a) {
   const unsigned long long eh = block_excl_1024(th, &tot_h);
   if (d < nd) {
     a.off_a[d] = ec;
-    a.cur_a[d] = ec;
+    a.cur_a[d] = (unsigned)ec;
     a.tpref_b[d] = eb;
     a.tpref_h[d] = eh;
     if (a.dB == 0) a.boff[d] = ec;
@@ -202,7 +202,7 @@ __global__ void __launch_bounds__(256) bucket_scan_b_kernel(BucketArgs a) {
     const unsigned d = threadIdx.x * kPer + i;
     if (d < nb) {
       a.boff[b0 + d] = run;
-      a.cur_b[b0 + d] = run;
+      a.cur_b[b0 + d] = (unsigned)run;
     }
     run += v[i];
   }
@@ -235,35 +235,44 @@ static_assert(kHistPassTiles * kPTile == kBucketHistTile && kHistPassTiles <= 25
 
 template <int RB>
 constexpr size_t bpart_smem() {
-  return (size_t)(kPTile + 2) * 8 + (size_t)(1 << RB) * (4 + 4 + 8);
+  return (size_t)(kPTile + 2) * 8 + (size_t)(1 << RB) * (4 + 4);
 }
 
 // H32: the cell field has at most 32 bits, so h is computed in 32-bit
 // arithmetic (the product modulo 2^cb depends only on the low 32 bits of each
 // factor).
-// 4 blocks per SM, without spills (5 blocks, 48 registers, spill in both passes)
+// The pass is bound by shared memory (its wavefronts keep the data pipe 65-75 %
+// busy: rank atomics and offset gathers at random digits, the scatter of 8-byte
+// keys), so a tile is read from it once and its keys stay in registers until the
+// scatter, with digit and rank in one word (recomputing the digit spilled and took
+// 8 % longer); destinations are 32-bit (a bucketed buffer has fewer than 2^32 keys) and
+// a key with bit 63 is padding.  290 M keys of the 4096 x 256 random affine model:
+// 9-bit pass A 1.06 ms (1.17 with one 64-bit claim per digit), 8-bit pass B
+// 1.01 ms (1.07).  Loading the tile straight into registers was slower (pass B
+// 1.25 ms: the loads in flight need L1 lines), as were 3 and 5 blocks per SM.
 template <int RB, bool B, bool H32>
 __global__ void __launch_bounds__(kPThreads, 4) bucket_partition_kernel(BucketArgs a) {
   constexpr int R = 1 << RB;
-  constexpr int DPT = (R + kPThreads - 1) / kPThreads;
+  constexpr int DPT = R > kPThreads ? R / kPThreads : 1;   // digits per thread (consecutive)
   constexpr int kWarps = kPThreads / 32;
+  constexpr unsigned kNone = ~0u;
   extern __shared__ __align__(16) unsigned char smem[];
-  uint64_t* s_keys = reinterpret_cast<uint64_t*>(smem);                            // [kPTile + 2]
-  unsigned int* cnt = reinterpret_cast<unsigned int*>(s_keys + kPTile + 2);       // [R]
-  unsigned int* excl = cnt + R;                                                     // [R]
-  unsigned long long* delta = reinterpret_cast<unsigned long long*>(excl + R);      // [R]
+  uint64_t* s_keys = reinterpret_cast<uint64_t*>(smem);                        // [kPTile + 2]
+  unsigned int* cnt = reinterpret_cast<unsigned int*>(s_keys + kPTile + 2);    // [R] counts, then tile offsets
+  unsigned int* delta = cnt + R;                                               // [R] output position - tile position
   __shared__ unsigned int s_wt[kWarps];
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
 
   // tile geometry (block-uniform)
-  uint64_t t0, len;
+  uint64_t t0;
+  unsigned len;
   unsigned long long* cursor;
   uint32_t sh, dbits;
   if (!B) {
     t0 = (uint64_t)blockIdx.x * kPTile;
     if (t0 >= a.n) return;
-    len = min((uint64_t)kPTile, a.n - t0);
-    cursor = a.cur_a;
+    len = (unsigned)min((uint64_t)kPTile, a.n - t0);
+    cursor = reinterpret_cast<unsigned long long*>(a.cur_a);
     sh = a.cb - a.dA;
     dbits = a.dA;
   } else {
@@ -273,12 +282,12 @@ __global__ void __launch_bounds__(kPThreads, 4) bucket_partition_kernel(BucketAr
     const uint32_t d1 = a.tile_a[t];
     // (every entry below tpref_b[nd] was written by the histogram of this check)
     if (d1 >= nd) {
-      if (threadIdx.x == 0) atomicOr(a.err, (unsigned int)kErrSortRange);
+      if (tid == 0) atomicOr(a.err, (unsigned int)kErrSortRange);
       return;
     }
     t0 = a.off_a[d1] + (t - a.tpref_b[d1]) * kPTile;
-    len = min((uint64_t)kPTile, (uint64_t)(a.off_a[d1 + 1] - t0));
-    cursor = a.cur_b + ((uint64_t)d1 << a.dB);
+    len = (unsigned)min((uint64_t)kPTile, (uint64_t)(a.off_a[d1 + 1] - t0));
+    cursor = reinterpret_cast<unsigned long long*>(a.cur_b + ((uint64_t)d1 << a.dB));   // (dB >= 1)
     sh = a.cb - a.dA - a.dB;
     dbits = a.dB;
   }
@@ -289,19 +298,19 @@ __global__ void __launch_bounds__(kPThreads, 4) bucket_partition_kernel(BucketAr
     return (unsigned)(cell_hash_of(k >> cs, a.cmask) >> sh) & dmask;
   };
 
-  for (int i = threadIdx.x; i < R; i += kPThreads) cnt[i] = 0;
+  for (int i = tid; i < R; i += kPThreads) cnt[i] = 0;
   // the tile into shared memory by 16-byte copies where it can be: a full tile
   // of a 16-byte aligned buffer at an even key position, or at an odd one
   // widened by a key on each side (kept inside the buffer: the key after the
   // tile exists); else 8-byte copies.  Key j of the tile is s_keys[off + j].
-  const bool full = len == (uint64_t)kPTile;
+  const bool full = len == (unsigned)kPTile;
   const bool al16 = (reinterpret_cast<uintptr_t>(a.keys_in) & 15u) == 0u;
   int off = 0;
   __shared__ __align__(8) unsigned long long s_bar;
   if (kPartBulkCopy && B && full && al16 && ((t0 & 1u) == 0u || t0 + kPTile < a.n)) {
     // one bulk copy by the TMA engine (the widened tile for an odd start)
     off = (int)(t0 & 1u);
-    if (threadIdx.x == 0) {
+    if (tid == 0) {
       mbar_init(&s_bar, 1u);
       bulk_load(s_keys, a.keys_in + (t0 - (uint64_t)off), (unsigned)((kPTile + 2 * off) * 8), &s_bar);
     }
@@ -310,27 +319,31 @@ __global__ void __launch_bounds__(kPThreads, 4) bucket_partition_kernel(BucketAr
   } else if (full && al16 && (t0 & 1u) == 0u) {
 #pragma unroll
     for (int m = 0; m < kPTile / 2 / kPThreads; ++m) {
-      const int j = m * kPThreads + (int)threadIdx.x;
+      const int j = m * kPThreads + tid;
       cp_async16(s_keys + 2 * j, a.keys_in + t0 + 2 * j);
     }
   } else if (full && al16 && t0 + kPTile < a.n) {
     off = 1;
-    for (int j = threadIdx.x; j < kPTile / 2 + 1; j += kPThreads)
+    for (int j = tid; j < kPTile / 2 + 1; j += kPThreads)
       cp_async16(s_keys + 2 * j, a.keys_in + (t0 - 1) + 2 * j);
   } else {
-    for (int j = threadIdx.x; j < (int)len; j += kPThreads) cp_async8(s_keys + j, a.keys_in + t0 + j);
+    for (int j = tid; j < (int)len; j += kPThreads) cp_async8(s_keys + j, a.keys_in + t0 + j);
   }
   cp_async_wait_all();
   __syncthreads();
-
-  const int lpos = w * (32 * kPItems) + lane;
-  unsigned short r[kPItems];   // rank inside the digit (0xffff: no key)
+  uint64_t k[kPItems];
 #pragma unroll
   for (int i = 0; i < kPItems; ++i) {
-    const int j = lpos + i * 32;
-    const uint64_t k = j < (int)len ? s_keys[off + j] : kSentinel;
-    const bool valid = j < (int)len && (B || k != kSentinel);
-    const unsigned d = valid ? digit(k) : 0u;
+    const unsigned j = (unsigned)(i * kPThreads + tid);
+    k[i] = j < len ? s_keys[off + j] : kSentinel;
+  }
+  // rank inside the digit: one shared atomic per key, one per warp when the warp
+  // holds one digit
+  unsigned dr[kPItems];   // digit << 16 | rank, kNone: no key
+#pragma unroll
+  for (int i = 0; i < kPItems; ++i) {
+    const bool valid = (int)(uint32_t)(k[i] >> 32) >= 0;   // (keys have 63 bits)
+    const unsigned d = digit(k[i]);
     const unsigned d0 = __shfl_sync(FULL, d, 0);
     unsigned rank = 0;
     if (__all_sync(FULL, valid && d == d0)) {
@@ -340,56 +353,80 @@ __global__ void __launch_bounds__(kPThreads, 4) bucket_partition_kernel(BucketAr
     } else if (valid) {
       rank = atomicAdd(&cnt[d], 1u);
     }
-    r[i] = valid ? (unsigned short)rank : (unsigned short)0xffffu;
+    dr[i] = valid ? (d << 16) | rank : kNone;
   }
   __syncthreads();
-  // per digit: claim the output range, tile offsets
-  unsigned carry = 0;
+  // Per digit the output range is claimed and the tile offset scanned.  Pass A's
+  // tiles all claim from the same few cache lines, and those atomics bound it
+  // (their L2 slices were busy while the others idled): two digits share a 64-bit
+  // atomic, and a warp's claims lie side by side.  The scan takes consecutive
+  // digits per thread instead, while the claims are on their way.
+  constexpr int PPT = R / 2 > kPThreads ? R / 2 / kPThreads : 1;   // digit pairs per thread
+  unsigned long long claim[PPT];
+#pragma unroll
+  for (int q = 0; q < PPT; ++q) {
+    const int pr = q * kPThreads + tid;
+    claim[q] = 0;
+    if (pr < R / 2) {
+      const unsigned long long c = (unsigned long long)cnt[2 * pr] | ((unsigned long long)cnt[2 * pr + 1] << 32);
+      if (c) claim[q] = atomicAdd(&cursor[pr], c);
+    }
+  }
+  unsigned sum = 0;
+#pragma unroll
+  for (int q = 0; q < DPT; ++q)
+    if (tid * DPT + q < R) sum += cnt[tid * DPT + q];
+  unsigned x = sum;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const unsigned y = __shfl_up_sync(FULL, x, o);
+    if (lane >= o) x += y;
+  }
+  if (lane == 31) s_wt[w] = x;
+  __syncthreads();
+  unsigned run = x - sum, total = 0;
+#pragma unroll
+  for (int i = 0; i < kWarps; ++i) {
+    if (i < w) run += s_wt[i];
+    total += s_wt[i];
+  }
 #pragma unroll
   for (int q = 0; q < DPT; ++q) {
-    const int dg = q * kPThreads + threadIdx.x;
-    const unsigned c = dg < R ? cnt[dg] : 0u;
-    const unsigned long long claim = c ? atomicAdd(&cursor[dg], (unsigned long long)c) : 0ull;
-    unsigned x = c;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const unsigned y = __shfl_up_sync(FULL, x, o);
-      if (lane >= o) x += y;
-    }
-    if (lane == 31) s_wt[w] = x;
-    __syncthreads();
-    unsigned base = carry, tot = 0;
-    for (int i = 0; i < kWarps; ++i) {
-      if (i < w) base += s_wt[i];
-      tot += s_wt[i];
-    }
-    __syncthreads();
+    const int dg = tid * DPT + q;
     if (dg < R) {
-      const unsigned e = base + x - c;
-      excl[dg] = e;
-      delta[dg] = claim - e;
+      const unsigned c = cnt[dg];
+      cnt[dg] = run;
+      run += c;
     }
-    carry += tot;
   }
   __syncthreads();
-  uint64_t kk[kPItems];
 #pragma unroll
-  for (int i = 0; i < kPItems; ++i) {
-    const int j = lpos + i * 32;
-    kk[i] = j < (int)len ? s_keys[off + j] : kSentinel;
+  for (int q = 0; q < PPT; ++q) {
+    const int pr = q * kPThreads + tid;
+    if (pr < R / 2) {
+      delta[2 * pr] = (unsigned)claim[q] - cnt[2 * pr];
+      delta[2 * pr + 1] = (unsigned)(claim[q] >> 32) - cnt[2 * pr + 1];
+    }
   }
-  __syncthreads();   // every key read before any is overwritten
+  // the keys in digit order
 #pragma unroll
   for (int i = 0; i < kPItems; ++i)
-    if (r[i] != 0xffffu) s_keys[excl[digit(kk[i])] + r[i]] = kk[i];
+    if (dr[i] != kNone) s_keys[cnt[dr[i] >> 16] + (dr[i] & 0xffffu)] = k[i];
   __syncthreads();
-  // carry = valid keys of the tile
-  for (int pos = threadIdx.x; pos < (int)carry; pos += kPThreads) {
+  // and out, consecutive keys of a digit to consecutive addresses; in range
+  // whenever the histogram and the ranks agree (see sort.cu)
+  const unsigned n = (unsigned)a.n;
+  auto put = [&](unsigned pos) {
     const uint64_t key = s_keys[pos];
-    const unsigned long long dst = delta[digit(key)] + (unsigned long long)pos;
-    // in range whenever the histogram and the ranks agree (see sort.cu)
-    if (dst < a.n) a.keys_out[dst] = key;
+    const unsigned dst = delta[digit(key)] + pos;
+    if (dst < n) a.keys_out[dst] = key;
     else atomicOr(a.err, (unsigned int)kErrSortRange);
+  };
+  if (total == (unsigned)kPTile) {
+#pragma unroll 8
+    for (int i = 0; i < kPItems; ++i) put((unsigned)(i * kPThreads + tid));
+  } else {
+    for (unsigned pos = tid; pos < total; pos += kPThreads) put(pos);
   }
 }
 

@@ -161,13 +161,13 @@ struct BucketArgs {
   uint32_t dA, dB;
   unsigned long long* hist_a;       // [2^dA] valid keys per A-bucket
   unsigned long long* off_a;        // [2^dA + 1] A-bucket offsets (exclusive, then the total)
-  unsigned long long* cur_a;        // [2^dA] pass-A output cursors
+  unsigned* cur_a;                  // [2^dA] pass-A output cursors (two digits are claimed by one 64-bit atomic)
   unsigned long long* tpref_b;      // [2^dA + 1] pass-B tiles before each A-bucket
   unsigned* tile_a;                 // [pass-B tiles] the A-bucket of each pass-B tile (written by the histogram)
   unsigned long long* tpref_h;      // [2^dA + 1] histogram tiles before each A-bucket
   unsigned long long* hist_b;       // [2^D] keys per bucket
   unsigned long long* boff;         // [2^D + 1] bucket offsets
-  unsigned long long* cur_b;        // [2^D] pass-B output cursors
+  unsigned* cur_b;                  // [2^D] pass-B output cursors
   unsigned int* err;
 };
 cudaError_t launch_bucket_hist_a(const BucketArgs& a, cudaStream_t st);

@@ -282,7 +282,7 @@ bool plan_buckets(uint64_t n, uint64_t n_expect, uint32_t cb, uint32_t phase_bit
   bp->off_a = off;
   off = align256(off + (na + 1) * 8);
   bp->cur_a = off;
-  off = align256(off + na * 8);
+  off = align256(off + na * 4);
   bp->tpref_b = off;
   off = align256(off + (na + 1) * 8);
   bp->tile_a = off;
@@ -292,7 +292,7 @@ bool plan_buckets(uint64_t n, uint64_t n_expect, uint32_t cb, uint32_t phase_bit
   bp->boff = off;
   off = align256(off + (nb + 1) * 8);
   bp->cur_b = off;
-  off = align256(off + nb * 8);
+  off = align256(off + nb * 4);
   bp->end = off;
   return true;
 }
@@ -467,13 +467,13 @@ rc_status enqueue_bucketed(const rc::WorkspacePlan& p, uint8_t* ws, uint64_t* bu
   a.dB = bp.dB;
   a.hist_a = u64(bp.hist_a);
   a.off_a = u64(bp.off_a);
-  a.cur_a = u64(bp.cur_a);
+  a.cur_a = reinterpret_cast<unsigned*>(ws + bp.cur_a);
   a.tpref_b = u64(bp.tpref_b);
   a.tile_a = reinterpret_cast<unsigned*>(ws + bp.tile_a);
   a.tpref_h = u64(bp.tpref_h);
   a.hist_b = u64(bp.hist_b);
   a.boff = u64(bp.boff);
-  a.cur_b = u64(bp.cur_b);
+  a.cur_b = reinterpret_cast<unsigned*>(ws + bp.cur_b);
   a.err = sa.err;
   uint64_t* fin = buf0;
   uint64_t* scratch = buf1;
