@@ -227,52 +227,188 @@ struct Gen {
     }
   }
 
-  std::string row(int r) {
+  // -------------------------------------------------------------------------
+  // Value ranges.  Every row of a statement is bounded from the grid, the loop
+  // bounds, the divisors and the table values.  Rows whose values fit 32 bits are
+  // evaluated in 32-bit arithmetic (modulo 2^32 every partial result may wrap, the
+  // value itself does not), and checks that a range decides are left out.  A row
+  // without a bound (or one that might leave 64 bits) is evaluated as it is
+  // written, in 64 bits.
+  // -------------------------------------------------------------------------
+  struct Range {
+    __int128 lo = 0, hi = 0;
+    bool known = false;
+    bool narrow() const { return known && lo >= -2147483647 && hi <= 2147483647; }
+    bool inside(__int128 a, __int128 b) const { return known && lo >= a && hi < b; }   // [a, b)
+  };
+  std::vector<Range> r_it, r_term;   // the statement's iterators and terms
+  std::vector<bool> n_it, n_term;    // ... that are 32-bit variables
+
+  static Range bounded(__int128 lo, __int128 hi) {
+    Range r;
+    r.lo = lo;
+    r.hi = hi;
+    const __int128 lim = (__int128)1 << 62;
+    r.known = lo >= -lim && hi <= lim;
+    return r;
+  }
+  Range range(int r) const {
+    const Row& R = rows[r];
+    __int128 lo = R.c0, hi = R.c0;
+    const __int128 lim = (__int128)1 << 62;
+    auto add = [&](int64_t c, __int128 l, __int128 h) {   // (|c| < 2^64, |l|, |h| <= 2^62: no overflow)
+      lo += c >= 0 ? c * l : c * h;
+      hi += c >= 0 ? c * h : c * l;
+    };
+    for (int i = 0; i < 6; ++i) {
+      if (!R.ct[i]) continue;
+      const uint32_t n = i < 3 ? m.host.block[i] : m.host.grid[i - 3];
+      add(R.ct[i], 0, (__int128)n - 1);
+      if (lo < -lim || hi > lim) return Range();
+    }
+    for (int k = 0; k < R.nnz; ++k) {
+      const LinTerm& t = lin[R.off + k];
+      const Range& v = t.var < kMaxLoops ? r_it[t.var] : r_term[t.var - kMaxLoops];
+      if (!v.known) return Range();
+      add(t.coef, v.lo, v.hi);
+      if (lo < -lim || hi > lim) return Range();
+    }
+    return bounded(lo, hi);
+  }
+  static __int128 fdiv128(__int128 a, int64_t d) { return a >= 0 ? a / d : -((-a + d - 1) / d); }
+  Range term_range(const Term& T) const {
+    const Range a = range(T.row);
+    if (T.op == kLoad) {
+      const uint64_t* tidx = reinterpret_cast<const uint64_t*>(img + m.sec_tabidx);
+      const int64_t* data = reinterpret_cast<const int64_t*>(img + m.sec_tdata) + tidx[2 * T.d];
+      const uint64_t n = tidx[2 * T.d + 1];
+      int64_t lo = 0, hi = 0;   // (a load outside the table is 0)
+      for (uint64_t i = 0; i < n; ++i) {
+        lo = std::min(lo, data[i]);
+        hi = std::max(hi, data[i]);
+      }
+      return bounded(lo, hi);
+    }
+    if (T.op == kFdiv) return a.known ? bounded(fdiv128(a.lo, T.d), fdiv128(a.hi, T.d)) : Range();
+    return a.inside(0, T.d) ? a : bounded(0, (__int128)T.d - 1);
+  }
+  // the ranges of a statement's iterators and terms, outer levels first
+  void find_ranges(const DevStmt& S) {
+    r_it.assign(kMaxLoops, Range());
+    r_term.assign(kMaxTerms, Range());
+    n_it.assign(kMaxLoops, false);
+    n_term.assign(kMaxTerms, false);
+    for (int l = 0; l <= S.n_loops; ++l) {
+      for (int q = 0; q < S.n_terms; ++q)
+        if (terms[S.term0 + q].level == l) {
+          r_term[q] = term_range(terms[S.term0 + q]);
+          n_term[q] = r_term[q].narrow();
+        }
+      if (l == S.n_loops) break;
+      const Range lo = range(S.row_lower[l]), hi = range(S.row_upper[l]);
+      if (!lo.known || !hi.known) continue;
+      r_it[l] = bounded(lo.lo, std::max(hi.hi - 1, lo.lo));
+      // (the variable itself runs past the upper bound by a step at most)
+      n_it[l] = lo.narrow() && hi.narrow() && S.step[l] < (1ll << 30) && hi.hi + S.step[l] <= 2147483647 && r_it[l].narrow();
+    }
+  }
+
+  // a row in 64 bits, wrapping (so in unsigned arithmetic: the compiler may take
+  // signed values for bounded)
+  std::string row64(int r) {
     static const char* tv[6] = {"tx", "ty", "tz", "bx", "by", "bz"};
     const Row& R = rows[r];
-    std::string e = lit(R.c0);
+    std::string e = ulit((uint64_t)R.c0);
     for (int i = 0; i < 6; ++i)
-      if (R.ct[i]) e += " + " + lit(R.ct[i]) + " * " + tv[i];
+      if (R.ct[i]) e += " + " + ulit((uint64_t)R.ct[i]) + " * (unsigned long long)" + tv[i];
     for (int k = 0; k < R.nnz; ++k) {
       const LinTerm& t = lin[R.off + k];
       const std::string v = t.var < kMaxLoops ? "i" + std::to_string(t.var) : "q" + std::to_string(t.var - kMaxLoops);
-      e += " + " + lit(t.coef) + " * " + v;
+      e += " + " + ulit((uint64_t)t.coef) + " * (unsigned long long)" + v;
     }
-    return "(" + e + ")";
+    return "((long long)(" + e + "))";
   }
+  // its value modulo 2^32
+  std::string row32(int r) {
+    static const char* tv[6] = {"tx", "ty", "tz", "bx", "by", "bz"};
+    const Row& R = rows[r];
+    auto u = [](int64_t v) { return std::to_string((uint32_t)(uint64_t)v) + "u"; };
+    std::string e = u(R.c0);
+    for (int i = 0; i < 6; ++i)
+      if (R.ct[i]) e += " + " + u(R.ct[i]) + " * (unsigned)" + tv[i];
+    for (int k = 0; k < R.nnz; ++k) {
+      const LinTerm& t = lin[R.off + k];
+      const std::string v = t.var < kMaxLoops ? "i" + std::to_string(t.var) : "q" + std::to_string(t.var - kMaxLoops);
+      e += " + " + u(t.coef) + " * (unsigned)" + v;
+    }
+    return "((int)(" + e + "))";
+  }
+  std::string row(int r) { return range(r).narrow() ? row32(r) : row64(r); }
+  std::string row_type(int r) { return range(r).narrow() ? "int" : "long long"; }
 
   void emit_terms(const DevStmt& S, int level, const std::string& ind) {
     for (int q = 0; q < S.n_terms; ++q) {
       const Term& T = terms[S.term0 + q];
       if (T.level != level) continue;
-      const std::string a = row(T.row);
+      const Range a = range(T.row);
+      const bool small_d = T.d < (1ll << 31);
       std::string v;
       if (T.op == kLoad) {
         const uint64_t* tidx = reinterpret_cast<const uint64_t*>(img + m.sec_tabidx);
-        v = "tload_c(tdata, " + ulit(tidx[2 * T.d]) + ", " + ulit(tidx[2 * T.d + 1]) + ", " + a + ")";
-      } else if (T.op == kFdiv) {
-        v = is_pow2(T.d) ? "(" + a + " >> " + std::to_string(log2i(T.d)) + ")" : "fdiv_c(" + a + ", " + lit(T.d) + ")";
+        v = "tload_c(tdata, " + ulit(tidx[2 * T.d]) + ", " + ulit(tidx[2 * T.d + 1]) + ", (long long)" + row(T.row) + ")";
+      } else if (T.op == kMod && a.inside(0, T.d)) {
+        v = row(T.row);
+      } else if (is_pow2(T.d) && (!a.narrow() || small_d)) {
+        v = T.op == kFdiv ? "(" + row(T.row) + " >> " + std::to_string(log2i(T.d)) + ")"
+                          : "(" + row(T.row) + " & " + (a.narrow() ? std::to_string(T.d - 1) : lit(T.d - 1)) + ")";
+      } else if (a.narrow() && small_d) {
+        const std::string d = std::to_string(T.d);
+        if (a.lo >= 0) v = "(int)((unsigned)" + row32(T.row) + (T.op == kFdiv ? " / " : " % ") + d + "u)";
+        else v = (T.op == kFdiv ? "fdiv_n(" : "mod_n(") + row32(T.row) + ", " + d + ")";
       } else {
-        v = is_pow2(T.d) ? "(" + a + " & " + lit(T.d - 1) + ")" : "mod_c(" + a + ", " + lit(T.d) + ")";
+        v = (T.op == kFdiv ? "fdiv_c(" : "mod_c(") + row64(T.row) + ", " + lit(T.d) + ")";
       }
-      o << ind << "const long long q" << q << " = " << v << ";\n";
+      o << ind << "const " << (n_term[q] ? "int" : "long long") << " q" << q << " = "
+        << (n_term[q] ? "(int)" : "(long long)") << v << ";\n";
     }
+  }
+
+  // whether a row keeps its value while only the innermost iterator moves
+  bool fixed_inside(const DevStmt& S, int r) const {
+    for (int k = 0; k < rows[r].nnz; ++k) {
+      const LinTerm& t = lin[rows[r].off + k];
+      if (t.var < kMaxLoops ? t.var == S.n_loops - 1 : terms[S.term0 + t.var - kMaxLoops].level == S.n_loops) return false;
+    }
+    return true;
   }
 
   void emit_stmt(uint32_t s) {
     const DevStmt& S = stmts[s];
-    const uint64_t T = m.host.n_threads;
+    const DevModel& h = m.host;
+    const uint64_t T = h.n_threads;
+    find_ranges(S);
     o << "    case " << s << ": {\n";
     const bool distinct = !dp[s].point.empty();
     if (chunked) {
       // keys go to chunk_put; no slots
     } else if (S.dense) {
-      o << "      unsigned long long slot = (all_points ? " << ulit(S.slot_base) << " : " << ulit(check_base[s])
+      o << "      unsigned long long* out = keys + (all_points ? " << ulit(S.slot_base) << " : " << ulit(check_base[s])
         << ") + g;\n";
     } else {
-      o << "      unsigned long long off = unit_offset[" << ulit(S.slot_base) << " + g]"
+      o << "      unsigned long long* out = keys + unit_offset[" << ulit(S.slot_base) << " + g]"
         << (check_dense != h_dense() ? " - (all_points ? 0ull : " + ulit(h_dense() - check_dense) + ")" : std::string())
         << ";\n";
+    }
+    // An access that stays where it is while the innermost loop runs repeats its
+    // last key there (the same instance again): only the first is kept.
+    std::vector<bool> repeats(S.n_acc, false);
+    for (int a = 0; a < S.n_acc && S.n_loops > 0 && !distinct; ++a) {
+      const DevAccess& A = accs[S.acc0 + a];
+      if (A.key_idx < 0) continue;
+      bool fixed = fixed_inside(S, S.row_phase) && (S.row_wphase < 0 || fixed_inside(S, S.row_wphase));
+      for (int d = 0; d < A.ndims; ++d) fixed = fixed && fixed_inside(S, A.row0 + d);
+      repeats[a] = fixed;
+      if (fixed) o << "      unsigned long long last" << a << " = ~0ull;\n";
     }
     emit_terms(S, 0, "      ");
     std::string ind = "      ";
@@ -283,98 +419,148 @@ struct Gen {
       ind += "  ";
       o << ind << "unsigned e = " << (chunked ? "" : "all_points ? p : ") << "(unsigned)pts" << s << "[p].x;\n";
       for (int l = S.n_loops - 1; l >= 0; --l) {
-        o << ind << "const long long i" << l << " = " << row(S.row_lower[l]) << " + " << lit(S.step[l])
-          << " * (long long)(e" << (l ? " % " + std::to_string(S.trips[l]) + "u" : std::string()) << ");\n";
+        const std::string k = "(e" + (l ? " % " + std::to_string(S.trips[l]) + "u" : std::string()) + ")";
+        if (n_it[l])
+          o << ind << "const int i" << l << " = " << row32(S.row_lower[l]) << " + " << S.step[l] << " * (int)" << k << ";\n";
+        else
+          o << ind << "const long long i" << l << " = " << row64(S.row_lower[l]) << " + " << lit(S.step[l])
+            << " * (long long)" << k << ";\n";
         if (l) o << ind << "e /= " << S.trips[l] << "u;\n";
       }
       for (int l = 0; l < S.n_loops; ++l) emit_terms(S, l + 1, ind);
     }
     for (int l = 0; l < S.n_loops && !distinct; ++l) {
-      o << ind << "for (long long i" << l << " = " << row(S.row_lower[l]) << "; i" << l << " < " << row(S.row_upper[l])
-        << "; i" << l << " += " << lit(S.step[l]) << ") {\n";
+      if (n_it[l])
+        o << ind << "for (int i" << l << " = " << row32(S.row_lower[l]) << "; i" << l << " < " << row32(S.row_upper[l])
+          << "; i" << l << " += " << S.step[l] << ") {\n";
+      else
+        o << ind << "for (long long i" << l << " = " << row64(S.row_lower[l]) << "; i" << l << " < "
+          << row64(S.row_upper[l]) << "; i" << l << " += " << lit(S.step[l]) << ") {\n";
       ind += "  ";
       emit_terms(S, l + 1, ind);
     }
-    // guards
+    // guards (those that the ranges decide left out)
     std::string gcond = "true";
-    for (int gi = 0; gi < S.n_guards; ++gi) gcond += " && " + row(S.guard_row0 + gi) + " >= 0";
+    for (int gi = 0; gi < S.n_guards; ++gi) {
+      const Range r = range(S.guard_row0 + gi);
+      if (r.known && r.lo >= 0) continue;
+      gcond += " && " + row(S.guard_row0 + gi) + " >= 0";
+    }
     o << ind << "if (" << gcond << ") {\n";
     const std::string in2 = ind + "  ";
-    const bool fine = S.row_wphase >= 0 || m.host.n_wphases > 1;
+    const bool fine = S.row_wphase >= 0 || h.n_wphases > 1;
+    // the (fine) interval; ph_ok: the ranges show that it is one
+    bool ph_ok = range(S.row_phase).inside(0, h.n_phases);
+    if (S.row_wphase >= 0) ph_ok = ph_ok && range(S.row_wphase).inside(0, h.n_wphases);
     if (fine) {
       // the fine interval phase * n_wphases + warp phase; -1 if either is out of range
       o << in2 << "const long long ph0 = " << row(S.row_phase) << ";\n";
       o << in2 << "const long long wph = " << (S.row_wphase >= 0 ? row(S.row_wphase) : std::string("0LL")) << ";\n";
-      o << in2 << "const long long ph = (ph0 < 0 || ph0 >= " << lit(m.host.n_phases) << " || wph < 0 || wph >= "
-        << lit(m.host.n_wphases) << ") ? -1LL : ph0 * " << lit(m.host.n_wphases) << " + wph;\n";
+      o << in2 << "const long long ph = (ph0 < 0 || ph0 >= " << lit(h.n_phases) << " || wph < 0 || wph >= "
+        << lit(h.n_wphases) << ") ? -1LL : ph0 * " << lit(h.n_wphases) << " + wph;\n";
     } else {
-      o << in2 << "const long long ph = " << row(S.row_phase) << ";\n";
+      o << in2 << "const " << row_type(S.row_phase) << " ph = " << row(S.row_phase) << ";\n";
     }
+    o << in2 << "(void)ph;\n";
+    const bool cl32 = m.total_cells < (1ull << 32);
     for (int a = 0; a < S.n_acc; ++a) {
       const DevAccess& A = accs[S.acc0 + a];
       const DevArray& arr = arrays[A.array];
+      bool sure = ph_ok, dims32 = true;   // every check decided; every index in 32 bits
+      for (int d = 0; d < A.ndims; ++d) {
+        const Range r = range(A.row0 + d);
+        sure = sure && r.inside(0, arr.ext[d]);
+        dims32 = dims32 && r.narrow();
+      }
+      if (sure && A.key_idx < 0) continue;   // an array never written, always in bounds: counted below
       o << in2 << "{\n";
       const std::string in3 = in2 + "  ";
-      for (int d = 0; d < A.ndims; ++d) o << in3 << "const long long v" << d << " = " << row(A.row0 + d) << ";\n";
-      o << in3 << "unsigned dc = 0xFFFFFFFFu;\n";
-      o << in3 << "if (ph < 0 || ph >= " << lit(m.host.n_phases * m.host.n_wphases) << ") dc = 0u;\n";
       for (int d = 0; d < A.ndims; ++d)
-        o << in3 << "else if (v" << d << " < 0 || v" << d << " >= " << lit(arr.ext[d]) << ") dc = " << d + 1 << "u;\n";
-      // row-major element index
-      std::string e;
+        o << in3 << "const " << row_type(A.row0 + d) << " v" << d << " = " << row(A.row0 + d) << ";\n";
+      if (!sure) {
+        o << in3 << "unsigned dc = 0xFFFFFFFFu;\n";
+        if (!ph_ok) o << in3 << "if (ph < 0 || ph >= " << lit(h.n_phases * h.n_wphases) << ") dc = 0u;\n" << in3 << "else\n";
+        for (int d = 0; d < A.ndims; ++d) {
+          const Range r = range(A.row0 + d);
+          if (r.inside(0, arr.ext[d])) continue;
+          if (r.narrow() && arr.ext[d] < (1ll << 31))
+            o << in3 << "if ((unsigned)v" << d << " >= " << arr.ext[d] << "u) dc = " << d + 1 << "u;\n" << in3 << "else\n";
+          else
+            o << in3 << "if (v" << d << " < 0 || v" << d << " >= " << lit(arr.ext[d]) << ") dc = " << d + 1 << "u;\n"
+              << in3 << "else\n";
+        }
+        o << in3 << "{ }\n";
+      }
+      // the linear cell, row-major (32-bit where every cell number is)
+      const bool c32 = cl32 && dims32;
+      std::string e = c32 ? std::to_string((uint32_t)arr.base) + "u" : ulit(arr.base);
       for (int d = 0; d < A.ndims; ++d) {
         int64_t stride = 1;
         for (int d2 = d + 1; d2 < A.ndims; ++d2) stride *= arr.ext[d2];
-        if (!e.empty()) e += " + ";
-        e += "v" + std::to_string(d) + " * " + lit(stride);
+        if (c32) e += " + (unsigned)v" + std::to_string(d) + " * " + std::to_string((uint32_t)stride) + "u";
+        else e += " + (unsigned long long)((long long)v" + std::to_string(d) + " * " + lit(stride) + ")";
       }
-      std::string cell = ulit(arr.base) + " + (unsigned long long)(" + e + ")";
-      if (arr.shared) cell += " + b * " + ulit(arr.cells);
+      if (arr.shared) e += c32 ? " + (unsigned)b * " + std::to_string((uint32_t)arr.cells) + "u" : " + b * " + ulit(arr.cells);
+      const std::string cell_t = c32 ? "unsigned" : "unsigned long long";
+      // the key's fields below the cell in one 32-bit word where they fit
+      const bool low32 = h.cell_shift <= 32 && ph_ok && !fine;
+      auto make = [&](const std::string& cl) {
+        const std::string c64 = "((unsigned long long)" + cl + " << " + std::to_string(h.cell_shift) + ")";
+        if (low32)
+          return c64 + " | (((unsigned)ph << " + std::to_string(h.phase_shift & 31u) + ") | (unsigned)low | " +
+                 std::to_string(A.kind) + "u)";
+        return c64 + " | ((unsigned long long)ph << " + std::to_string(h.phase_shift) + ") | low | " +
+               ulit((uint64_t)A.kind);
+      };
       const uint64_t pack = ((unsigned long long)s << 51) | ((unsigned long long)a << 45);
+      const std::string report = "atomicMin(oob, " + ulit(pack) + " | ((g & 0x3FFFFFFFFFFull) << 3) | dc);";
       if (chunked) {
         // the whole cell goes to the sink beside the key, whose cell field may not hold it
         o << in3 << "unsigned long long key = ~0ull, cl = ~0ull;\n";
-        o << in3 << "if (dc != 0xFFFFFFFFu) atomicMin(oob, " << ulit(pack) << " | ((g & 0x3FFFFFFFFFFull) << 3) | dc);\n";
-        o << in3 << "else { cl = " << cell << ";\n";
-        o << in3 << "  key = (cl << " << m.host.cell_shift << ") | ((unsigned long long)ph << " << m.host.phase_shift
-          << ") | low | " << ulit((uint64_t)A.kind) << "; }\n";
+        if (!sure) o << in3 << "if (dc != 0xFFFFFFFFu) " << report << "\n" << in3 << "else\n";
+        o << in3 << "{ cl = " << e << "; key = " << make("cl") << "; }\n";
         if (A.key_idx < 0) o << in3 << "(void)key; (void)cl;\n";
+        else if (repeats[a])   // (the cell tells the keys of a wide model apart, their cell field may not)
+          o << in3 << "if (cl != last" << a << ") chunk_put(a, key, cl);\n" << in3 << "last" << a << " = cl;\n";
         else o << in3 << "chunk_put(a, key, cl);\n";
         o << in2 << "}\n";
         continue;
       }
-      o << in3 << "unsigned long long key;\n";
-      o << in3 << "if (dc != 0xFFFFFFFFu) { atomicMin(oob, " << ulit(pack)
-        << " | ((g & 0x3FFFFFFFFFFull) << 3) | dc); key = ~0ull; }\n";
-      o << in3 << "else { const unsigned long long cl = " << cell << ";\n";
-      o << in3 << "  key = (cl >= cell_lo && cl < cell_hi && (part_mask == 0ull || ((cl * " << ulit(kCellHashMul)
-        << ") & part_mask) == part_val)) ? ((cl << " << m.host.cell_shift
-        << ") | ((unsigned long long)ph << " << m.host.phase_shift << ") | low | " << ulit((uint64_t)A.kind)
-        << ") : ~0ull; }\n";
       if (A.key_idx < 0) {
-        o << in3 << "(void)key;\n";   // array never written: checked, no key
-      } else {
-        // the pass-A histogram of the bucket path, counted as the keys are written
-        o << in3 << "if (hist_a != nullptr && key != ~0ull) atomicAdd(&hA[(unsigned)((((key >> "
-          << m.host.cell_shift << ") * " << ulit(kCellHashMul) << ") & hmask) >> hsh)], 1u);\n";
-        if (S.dense) o << in3 << "keys[slot + " << ulit((uint64_t)A.key_idx * T) << "] = key;\n";
-        else o << in3 << "keys[off + " << A.key_idx << "] = key;\n";
+        o << in3 << "if (dc != 0xFFFFFFFFu) " << report << "\n" << in2 << "}\n";   // checked, no key
+        continue;
       }
+      o << in3 << "unsigned long long key = ~0ull;\n";
+      if (!sure) o << in3 << "if (dc != 0xFFFFFFFFu) " << report << "\n" << in3 << "else\n";
+      o << in3 << "{\n" << in3 << "  const " << cell_t << " cl = " << e << ";\n";
+      o << in3 << "  if (!part_check || (cl >= cell_lo && cl < cell_hi && ((cl * " << ulit(kCellHashMul)
+        << ") & part_mask) == part_val)) key = " << make("cl") << ";\n";
+      if (repeats[a]) {
+        o << in3 << "  const unsigned long long now = key;\n";
+        o << in3 << "  if (!all_points && key == last" << a << ") key = ~0ull;\n" << in3 << "  last" << a << " = now;\n";
+      }
+      // the pass-A histogram of the bucket path, counted as the keys are written
+      o << in3 << "  if (hist_a != nullptr && key != ~0ull) atomicAdd(&hA["
+        << (c32 ? "((cl * " + std::to_string((uint32_t)kCellHashMul) + "u) & (unsigned)hmask) >> hsh"
+                : "(unsigned)(((cl * " + ulit(kCellHashMul) + ") & hmask) >> hsh)")
+        << "], 1u);\n" << in3 << "}\n";
+      if (S.dense) o << in3 << "out[" << ulit((uint64_t)A.key_idx * T) << "] = key;\n";
+      else o << in3 << "out[" << A.key_idx << "] = key;\n";
       o << in2 << "}\n";
     }
     if (!distinct) o << in2 << "cnt += " << S.n_acc << ";\n";
     else
       o << in2 << "cnt += " << S.n_acc << "u * (" << (chunked ? "" : "all_points ? 1u : ") << "(unsigned)pts" << s
         << "[p].y);\n";
-    if (!S.dense && !chunked) o << in2 << "off += " << S.n_key << ";\n";
+    if (!S.dense && !chunked) o << in2 << "out += " << S.n_key << ";\n";
     o << ind << "}";
     if (chunked) {
       o << "\n";
     } else if (S.dense) {
       o << " else {\n";
-      for (int kq = 0; kq < S.n_key; ++kq) o << in2 << "keys[slot + " << ulit((uint64_t)kq * T) << "] = ~0ull;\n";
+      for (int kq = 0; kq < S.n_key; ++kq) o << in2 << "out[" << ulit((uint64_t)kq * T) << "] = ~0ull;\n";
       o << ind << "}\n";
-      o << ind << "slot += " << ulit((uint64_t)S.n_key * T) << ";\n";
+      o << ind << "out += " << ulit((uint64_t)S.n_key * T) << ";\n";
     } else {
       o << "\n";
     }
@@ -392,6 +578,9 @@ struct Gen {
     o << "__device__ __forceinline__ long long fdiv_c(long long a, long long d) {\n"
          "  return a >= 0 ? a / d : -1 - (-(a + 1)) / d;\n}\n";
     o << "__device__ __forceinline__ long long mod_c(long long a, long long d) { return a - fdiv_c(a, d) * d; }\n";
+    o << "__device__ __forceinline__ int fdiv_n(int a, int d) {\n"
+         "  return a >= 0 ? (int)((unsigned)a / (unsigned)d) : -1 - (int)((unsigned)(-(a + 1)) / (unsigned)d);\n}\n"
+         "__device__ __forceinline__ int mod_n(int a, int d) { return a - fdiv_n(a, d) * d; }\n";
     o << "__device__ __forceinline__ long long tload_c(const long long* t, unsigned long long off, "
          "unsigned long long len, long long i) {\n"
          "  return (i < 0 || (unsigned long long)i >= len) ? 0LL : t[off + (unsigned long long)i];\n}\n";
@@ -462,6 +651,8 @@ struct Gen {
            "unsigned long long cell_lo, unsigned long long cell_hi, unsigned long long part_mask, unsigned long long part_val, "
            "const long long* __restrict__ tdata, "
            "unsigned long long* hist_a, unsigned long long hmask, unsigned hsh, unsigned hbins, unsigned units, unsigned all_points) {\n";
+      // a partial check (cell range or hash part); uniform
+      o << "  const bool part_check = cell_lo != 0ull || cell_hi != ~0ull || part_mask != 0ull;\n  (void)part_check;\n";
       o << "  __shared__ unsigned hA[" << kBucketMaxHistBins << "];\n";
       o << "  if (hist_a != nullptr) {\n"
            "    for (unsigned i = threadIdx.x; i < hbins; i += 128u) hA[i] = 0u;\n"
@@ -473,15 +664,25 @@ struct Gen {
                                                    "((unsigned long long)blockIdx.x * units + u)")
       << " * 128ull + threadIdx.x;\n";
     o << "  if (g < " << ulit(h.n_threads) << ") {\n";
-    o << "    const unsigned long long b = g / " << ulit(h.bs) << ";\n";
-    o << "    const unsigned t = (unsigned)(g - b * " << ulit(h.bs) << ");\n";
-    o << "    const long long tx = t % " << h.block[0] << "u, ty = (t / " << h.block[0] << "u) % " << h.block[1]
-      << "u, tz = t / " << (uint64_t)h.block[0] * h.block[1] << "u;\n";
-    o << "    const long long bx = (long long)(b % " << ulit(h.grid[0]) << "), by = (long long)((b / " << ulit(h.grid[0])
-      << ") % " << ulit(h.grid[1]) << "), bz = (long long)(b / " << ulit((uint64_t)h.grid[0] * h.grid[1]) << ");\n";
-    o << "    (void)tx; (void)ty; (void)tz; (void)bx; (void)by; (void)bz;\n";
+    if (h.n_threads < (1ull << 31)) {
+      // (every dimension is below 2^31 too)
+      o << "    const unsigned g32 = (unsigned)g, b32 = g32 / " << h.bs << "u, t = g32 - b32 * " << h.bs << "u;\n";
+      o << "    const int tx = t % " << h.block[0] << "u, ty = (t / " << h.block[0] << "u) % " << h.block[1]
+        << "u, tz = t / " << h.block[0] * h.block[1] << "u;\n";
+      o << "    const int bx = b32 % " << h.grid[0] << "u, by = (b32 / " << h.grid[0] << "u) % " << h.grid[1]
+        << "u, bz = b32 / " << h.grid[0] * h.grid[1] << "u;\n";
+      o << "    const unsigned long long b = b32;\n";
+    } else {
+      o << "    const unsigned long long b = g / " << ulit(h.bs) << ";\n";
+      o << "    const unsigned t = (unsigned)(g - b * " << ulit(h.bs) << ");\n";
+      o << "    const long long tx = t % " << h.block[0] << "u, ty = (t / " << h.block[0] << "u) % " << h.block[1]
+        << "u, tz = t / " << (uint64_t)h.block[0] * h.block[1] << "u;\n";
+      o << "    const long long bx = (long long)(b % " << ulit(h.grid[0]) << "), by = (long long)((b / " << ulit(h.grid[0])
+        << ") % " << ulit(h.grid[1]) << "), bz = (long long)(b / " << ulit((uint64_t)h.grid[0] * h.grid[1]) << ");\n";
+    }
+    o << "    (void)tx; (void)ty; (void)tz; (void)bx; (void)by; (void)bz; (void)b;\n";
     o << "    const unsigned long long low = (b << " << h.block_shift << ") | ((unsigned long long)t << "
-      << h.thread_shift << ");\n";
+      << h.thread_shift << ");\n    (void)low;\n";
     o << "    switch (blockIdx.y) {\n";
     for (uint32_t s = 0; s < h.n_stmts; ++s) emit_stmt(s);
     o << "    default: break;\n    }\n  }\n";

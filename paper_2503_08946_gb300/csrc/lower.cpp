@@ -741,6 +741,7 @@ rc_status lower_model(const rc_model_desc* d, Model* m, std::vector<int32_t>* ge
   m->sec_lin = off_lin;
   m->sec_terms = off_terms;
   m->sec_tabidx = off_tabidx;
+  m->sec_tdata = off_tdata;
   return RC_OK;
 }
 

@@ -429,7 +429,8 @@ struct Model {
   uint64_t coarse_tab = 0;        // fine interval q -> block interval (4 bits per q, q < 16)
   uint64_t grid_tab = 0;          // fine interval q -> grid interval (4 bits per q, q < 16)
   // sections of the program image (byte offsets), for the kernel generator
-  size_t sec_arrays = 0, sec_stmts = 0, sec_accs = 0, sec_rows = 0, sec_lin = 0, sec_terms = 0, sec_tabidx = 0;
+  size_t sec_arrays = 0, sec_stmts = 0, sec_accs = 0, sec_rows = 0, sec_lin = 0, sec_terms = 0, sec_tabidx = 0,
+         sec_tdata = 0;
   // grid interval (dense numbering) of every block interval, uint32 each: the
   // phase-sorted scan of models with warp or grid barriers and more than 16
   // fine intervals (0 = no such section)
