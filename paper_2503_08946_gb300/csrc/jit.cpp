@@ -154,6 +154,60 @@ struct Gen {
     lin = reinterpret_cast<const LinTerm*>(img + m.sec_lin);
     terms = reinterpret_cast<const Term*>(img + m.sec_terms);
     find_distinct_points();
+    plan_blocks();
+  }
+
+  // The slot kernel's blocks.  Every block counts the pass-A histogram of its keys
+  // in shared memory and adds it to the global one, whose few cache lines all
+  // blocks share: with a block per 128 threads and statement those additions took
+  // most of the time of statements with few keys per thread (the transposition,
+  // 12.6 M key slots: 77 us with 768 slots per block, 23 us with 7,000).  So a
+  // block takes as many 128-thread units of its statement as make about an equal
+  // share of the model's work: 10,000 keys (4,000 measured slower on models of 10
+  // to 50 M keys), in 12 to 64 blocks per SM (fewer leave SMs idle at the end;
+  // 4096 x 256: 0.60 ms with 16, 0.46 ms with 64), heavy statements first.
+  std::vector<uint32_t> blk_stmt, blk_first, blk_units;   // per statement, in launch order
+  uint64_t blocks = 0;
+  void plan_blocks() {
+    const uint32_t ns = m.host.n_stmts;
+    const uint64_t T = m.host.n_threads, units = (T + 127) / 128;
+    uint64_t general_keys = 0;
+    for (uint32_t s = 0; s < ns; ++s)
+      if (!stmts[s].dense) general_keys += stmts[s].n_key;
+    // keys per thread, an access without a key as half of one (points of
+    // statements with thread-dependent trips: their average)
+    std::vector<double> w(ns);
+    double total = 0;
+    for (uint32_t s = 0; s < ns; ++s) {
+      const DevStmt& S = stmts[s];
+      double pts = 16;
+      if (S.dense) pts = dp[s].point.empty() ? (double)S.n_iter : (double)dp[s].point.size();
+      else if (general_keys) pts = std::max(1.0, (double)m.host.general_slots / (double)(general_keys * T));
+      w[s] = pts * (S.n_key + 0.5 * (S.n_acc - S.n_key)) + 0.5;
+      total += w[s] * (double)units;
+    }
+    const double per_sm = std::min(64.0, std::max(12.0, total * 128.0 / (10000.0 * 152.0)));
+    double share = std::max(total / (152.0 * per_sm), 8.0);
+    std::vector<uint32_t> u(ns);
+    for (;; share *= 2) {
+      blocks = 0;
+      for (uint32_t s = 0; s < ns; ++s) {
+        const double n = share / w[s];
+        u[s] = n < 1 ? 1u : n > (double)units ? (uint32_t)std::min<uint64_t>(units, 1u << 30) : (uint32_t)n;
+        if (u[s] == 0) u[s] = 1;
+        blocks += (units + u[s] - 1) / u[s];
+      }
+      if (blocks <= 0x7fffffffull || units == 0) break;
+    }
+    blk_stmt.resize(ns);
+    for (uint32_t s = 0; s < ns; ++s) blk_stmt[s] = s;
+    std::stable_sort(blk_stmt.begin(), blk_stmt.end(), [&](uint32_t a, uint32_t b) { return w[a] * u[a] > w[b] * u[b]; });
+    uint64_t first = 0;
+    for (uint32_t s : blk_stmt) {
+      blk_first.push_back((uint32_t)first);
+      blk_units.push_back(u[s]);
+      first += (units + u[s] - 1) / u[s];
+    }
   }
 
   // The points of a dense statement's loop nest that differ in some row.  A
@@ -643,14 +697,17 @@ struct Gen {
       o << "extern \"C\" __global__ void __launch_bounds__(128) rc_chunk_jit(const ChunkJitArgs a) {\n";
       o << "  unsigned long long* oob = a.oob;\n  const long long* tdata = a.tdata;\n  (void)tdata;\n";
     } else {
-      // hist_a: the bucket path's pass-A digit counts (null: not counted here);
-      // each block expands `units` consecutive 128-thread units of its
-      // statement, so that its shared histogram is flushed once for them all
+      // hist_a: the bucket path's pass-A digit counts (null: not counted here).  The
+      // blocks of launch position i are [blk[i].x, blk[i + 1].x), each of blk[i].z
+      // consecutive 128-thread units of statement blk[i].y.
+      o << "__constant__ uint3 blk[" << h.n_stmts + 1 << "] = {";
+      for (uint32_t i = 0; i < h.n_stmts; ++i) o << "{" << blk_first[i] << "," << blk_stmt[i] << "," << blk_units[i] << "},";
+      o << "{" << blocks << ",0,1}};\n";
       o << "extern \"C\" __global__ void __launch_bounds__(128) rc_expand_jit(unsigned long long* __restrict__ keys, "
            "unsigned long long* oob, unsigned long long* inst, const unsigned long long* __restrict__ unit_offset, "
            "unsigned long long cell_lo, unsigned long long cell_hi, unsigned long long part_mask, unsigned long long part_val, "
            "const long long* __restrict__ tdata, "
-           "unsigned long long* hist_a, unsigned long long hmask, unsigned hsh, unsigned hbins, unsigned units, unsigned all_points) {\n";
+           "unsigned long long* hist_a, unsigned long long hmask, unsigned hsh, unsigned hbins, unsigned all_points) {\n";
       // a partial check (cell range or hash part); uniform
       o << "  const bool part_check = cell_lo != 0ull || cell_hi != ~0ull || part_mask != 0ull;\n  (void)part_check;\n";
       o << "  __shared__ unsigned hA[" << kBucketMaxHistBins << "];\n";
@@ -659,9 +716,14 @@ struct Gen {
            "    __syncthreads();\n  }\n";
     }
     o << "  unsigned long long cnt = 0;\n";
-    if (!chunked) o << "  for (unsigned u = 0; u < units; ++u) {\n";
+    if (!chunked)
+      o << "  unsigned bi = 0;\n  for (unsigned hi = " << h.n_stmts << "u; hi - bi > 1u;) {\n"
+           "    const unsigned mid = (bi + hi) >> 1;\n"
+           "    if (blk[mid].x <= blockIdx.x) bi = mid; else hi = mid;\n  }\n"
+           "  const unsigned stmt = blk[bi].y, units = blk[bi].z;\n"
+           "  for (unsigned u = 0; u < units; ++u) {\n";
     o << "  const unsigned long long g = " << (chunked ? "(unsigned long long)blockIdx.x" :
-                                                   "((unsigned long long)blockIdx.x * units + u)")
+                                                   "((unsigned long long)(blockIdx.x - blk[bi].x) * units + u)")
       << " * 128ull + threadIdx.x;\n";
     o << "  if (g < " << ulit(h.n_threads) << ") {\n";
     if (h.n_threads < (1ull << 31)) {
@@ -683,7 +745,7 @@ struct Gen {
     o << "    (void)tx; (void)ty; (void)tz; (void)bx; (void)by; (void)bz; (void)b;\n";
     o << "    const unsigned long long low = (b << " << h.block_shift << ") | ((unsigned long long)t << "
       << h.thread_shift << ");\n    (void)low;\n";
-    o << "    switch (blockIdx.y) {\n";
+    o << "    switch (" << (chunked ? "blockIdx.y" : "stmt") << ") {\n";
     for (uint32_t s = 0; s < h.n_stmts; ++s) emit_stmt(s);
     o << "    default: break;\n    }\n  }\n";
     if (!chunked) o << "  }\n";
@@ -774,7 +836,10 @@ bool jit_expand_build(Model* m) {
   }
   Gen g(*m);
   m->jit_fn = jit_compile(g.source(), "rc_expand_jit");
-  if (m->jit_fn) m->check_slots = g.check_dense + m->host.general_slots;
+  if (m->jit_fn) {
+    m->check_slots = g.check_dense + m->host.general_slots;
+    m->jit_blocks = (uint32_t)g.blocks;
+  }
   return m->jit_fn != nullptr;
 }
 
@@ -802,18 +867,9 @@ cudaError_t jit_expand_launch(const Model& m, uint64_t* keys, DevResult* res, cu
   unsigned long long hmask = eh ? eh->cmask : 0ull;
   unsigned hsh = eh ? eh->shift : 0u, hbins = eh ? eh->bins : 0u;
   if (hbins > (unsigned)kBucketMaxHistBins) return cudaErrorInvalidValue;
-  const uint64_t units_total = (m.host.n_threads + 127) / 128;
-  // with the histogram, blocks of up to kExpandHistUnits units (one flush per
-  // block), as long as the grid keeps about 64 blocks per SM
-  uint64_t units = 1;
-  if (eh) {
-    units = units_total * m.host.n_stmts / (152ull * 64ull);
-    units = units < 1 ? 1 : (units > kExpandHistUnits ? kExpandHistUnits : units);
-  }
-  unsigned units32 = (unsigned)units, all32 = all_points ? 1u : 0u;
-  void* params[] = {&keys, &oob, &inst, &uo, &lo, &hi, &pmask, &pval, &td, &hist, &hmask, &hsh, &hbins, &units32, &all32};
-  const unsigned gx = (unsigned)((units_total + units - 1) / units);
-  const CUresult r = dr.launch(fn, gx, m.host.n_stmts, 1, 128, 1, 1, 0, reinterpret_cast<CUstream>(st), params, nullptr);
+  unsigned all32 = all_points ? 1u : 0u;
+  void* params[] = {&keys, &oob, &inst, &uo, &lo, &hi, &pmask, &pval, &td, &hist, &hmask, &hsh, &hbins, &all32};
+  const CUresult r = dr.launch(fn, m.jit_blocks, 1, 1, 128, 1, 1, 0, reinterpret_cast<CUstream>(st), params, nullptr);
   return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorLaunchFailure;
 }
 

@@ -436,6 +436,7 @@ struct Model {
   // fine intervals (0 = no such section)
   size_t sec_gridof = 0;
   void* jit_fn = nullptr;         // generated expansion kernel (CUfunction), or null
+  uint32_t jit_blocks = 0;        // its blocks
   void* jit_chunk_fn = nullptr;   // wide models: generated count / route kernel, or null
   uint64_t max_iter_per_unit = 0;
 };
@@ -475,7 +476,6 @@ struct ExpandHist {
   uint32_t shift, bins;
 };
 constexpr int kBucketMaxHistBins = 1 << kBucketMaxDigitBits;
-constexpr unsigned kExpandHistUnits = 8;   // 128-thread units per block of a histogram-counting expansion
 // cells kept by a partial check: [lo, hi) and the hash part
 // ((c * kCellHashMul) & pmask) == pval (pmask = pval = 0: every part)
 struct CellFilter {
