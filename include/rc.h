@@ -350,7 +350,8 @@ enum { RC_OPT_STAGE_TIMES = 1, RC_OPT_GRAPH = 2, RC_OPT_CHUNKED = 4, RC_OPT_LSD 
  * scan; the result is identical to the radix-sorted check's.
  * RC_OPT_LSD (or a non-zero digit_bits, or any test flag) selects the stable
  * LSD radix sort followed by the ordered scan instead; other models of more
- * than 16 intervals, chunked checks and rc_sort_keys always take that path. */
+ * than 16 intervals, chunks that the cell test does not take, and rc_sort_keys
+ * always take that path. */
 
 typedef struct rc_inst {
   uint64_t block;          /* linear block index bx + gx*(by + gy*bz)             */

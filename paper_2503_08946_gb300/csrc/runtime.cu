@@ -792,6 +792,10 @@ void decode_result(const rc::DevResult& r, const rc::Model& m, rc_result* out, u
 // segment.  A cell races or not on its own, so the chunk counts add up and the
 // smallest racing pair is the one of the first chunk with a race.
 constexpr uint64_t kMaxChunkBuckets = 1ull << 20;
+// Buckets of a check whose workspace holds all keys at once: its chunks need not
+// be cut finely, and the host reads, scans and uploads a table of that many
+// counts (8 MB at 2^20: some 2 ms; 128 KB here).
+constexpr uint64_t kCoarseChunkBuckets = 1ull << 14;
 constexpr size_t kMaxChunks = 1u << 16;
 
 struct ChunkGeometry {
@@ -803,7 +807,9 @@ struct ChunkGeometry {
   size_t counts_off = 0, table_off = 0, chunks_off = 0, region_off = 0;
 };
 
-rc_status chunk_geometry(const rc::Model& m, const rc_check_opts* opts, ChunkGeometry* g) {
+rc_status chunk_geometry(const rc::Model& m, const rc_check_opts* opts, ChunkGeometry* g,
+                         uint64_t max_buckets = kMaxChunkBuckets) {
+  *g = ChunkGeometry();
   uint64_t lo = opts ? opts->cell_lo : 0;
   uint64_t hi = (opts && opts->cell_hi) ? opts->cell_hi : m.total_cells;
   if (hi > m.total_cells) hi = m.total_cells;
@@ -813,7 +819,7 @@ rc_status chunk_geometry(const rc::Model& m, const rc_check_opts* opts, ChunkGeo
   const uint32_t cb = m.host.cell_bits;
   g->max_span = cb >= 63 ? (1ull << 62) : (1ull << cb) - 1ull;
   uint32_t bs = 0;
-  while (bs < 63 && ((g->span + (1ull << bs) - 1) >> bs) > kMaxChunkBuckets) ++bs;
+  while (bs < 63 && ((g->span + (1ull << bs) - 1) >> bs) > max_buckets) ++bs;
   if (bs > 0 && (1ull << bs) > g->max_span) return RC_E_KEY_OVERFLOW;   // would need too many chunks
   g->bshift = bs;
   g->n_buckets = g->span ? ((g->span - 1) >> bs) + 1 : 0;
@@ -875,8 +881,15 @@ rc_status enqueue_chunked(rc_model* model, const rc_check_opts* opts, uint8_t* w
   rc_status s = chunk_geometry(m, opts, &g);
   if (s != RC_OK) return s;
   if (ws_bytes <= g.region_off) return RC_E_NOMEM;
-  const uint64_t cap = chunk_capacity(m, opts, ws_bytes - g.region_off, m.key_slots);
+  uint64_t cap = chunk_capacity(m, opts, ws_bytes - g.region_off, m.key_slots);
   if (cap == ~0ull) return RC_E_NOMEM;
+  if (cap >= m.key_slots) {
+    // (a bucket of at most a quarter of a chunk's span, so that the chunks stay few)
+    ChunkGeometry c;
+    if (chunk_geometry(m, opts, &c, kCoarseChunkBuckets) == RC_OK && c.region_off <= g.region_off &&
+        (1ull << c.bshift) <= c.max_span / 4)
+      g = c;
+  }
   uint8_t* region = ws + g.region_off;
   auto* counts = reinterpret_cast<unsigned long long*>(ws + g.counts_off);
   const rc::DevModel* dm = reinterpret_cast<const rc::DevModel*>(m.dev_program);
@@ -973,6 +986,7 @@ rc_status enqueue_chunked(rc_model* model, const rc_check_opts* opts, uint8_t* w
   uint64_t* keys0 = reinterpret_cast<uint64_t*>(region + pc.keys_off[0]);
   uint64_t* keys1 = reinterpret_cast<uint64_t*>(region + pc.keys_off[1]);
   const size_t K = chunks.size();
+  const bool bucket_ok = rc::bucket_path_allowed(opts) && rc::filter_allowed(m.sync_scopes, m.host.cell_shift);
   auto* c_lo = reinterpret_cast<const uint64_t*>(ws + g.chunks_off);
   for (const Wave& wv : waves) {
     if (s != RC_OK) break;
@@ -1004,6 +1018,8 @@ rc_status enqueue_chunked(rc_model* model, const rc_check_opts* opts, uint8_t* w
       jr.b0 = ra.b0;
       jr.n_buckets = ra.n_buckets;
       jr.low_mask = ra.low_mask;
+      jr.k0 = (uint32_t)wv.k0;
+      jr.nk = (uint32_t)(wv.k1 - wv.k0);
       s = cuda_status(rc::jit_chunk_launch(m, jr, st));
     } else if (s == RC_OK) {
       s = cuda_status(rc::launch_expand_route(dm, m.host.n_stmts, m.host.n_threads, m.has_deep_loops, ra, res, st));
@@ -1016,6 +1032,25 @@ rc_status enqueue_chunked(rc_model* model, const rc_check_opts* opts, uint8_t* w
       p.scan_warps = scan_warps_for(c.n);
       const uint32_t hi = m.host.cell_shift + std::max<uint32_t>(1u, rc::bit_length(c.span - 1));
       rc::plan_sort(m.host.sort_lo < hi ? m.host.sort_lo : hi, hi, opts ? opts->digit_bits : 0, &p.sort);
+      // the bucket path with the cell test, its section in the place of the radix
+      // sort's scratch (a chunk's keys hold no padding)
+      const uint32_t ccb = hi - m.host.cell_shift;
+      if (bucket_ok && c.n > 0 && m.host.cell_shift <= hi &&
+          rc::plan_buckets(c.n, c.n, ccb, m.host.phase_bits, true, pc.zero_lo, &p.bucket) && p.bucket.filter &&
+          p.bucket.end <= pc.long_off) {
+        s = cuda_status(rc::launch_init_check(res, k > wv.k0 ? 1u : 0u, nullptr, region + p.bucket.zero_lo,
+                                              p.bucket.zero_hi - p.bucket.zero_lo, nullptr, st));
+        rc::ScanArgs sa = scan_args(m, p, region, 0);
+        const uint64_t* fin = nullptr;
+        rc::FinishArgs fa;
+        if (s == RC_OK)
+          s = enqueue_bucketed(p, region, keys0 + c.base, keys1 + c.base, sa, st, &fin, &fa, nullptr, false, ccb);
+        sa.keys = fin;
+        if (s == RC_OK) s = cuda_status(rc::launch_bucket_witness(sa, fa, st));
+        if (s == RC_OK)
+          s = cuda_status(cudaMemcpyAsync(t->host + 1 + k, res, sizeof(rc::DevResult), cudaMemcpyDeviceToHost, st));
+        continue;
+      }
       // clear the digit histograms, the look-back words this chunk uses and the counters
       const size_t lb_used = (size_t)p.n_tiles * ((size_t)1 << rc::plan_max_bits(p.sort)) * 8;
       if (p.lookback_off + lb_used > pc.tilectr_off) s = RC_E_INVALID;   // cannot happen: sized for the widest digit
