@@ -128,6 +128,7 @@ int log2i(int64_t d) {
 struct DistinctPoints {
   std::vector<uint32_t> point, times;
 };
+constexpr unsigned kRouteChunks = 1024;            // chunks of a wave routed in two sweeps
 constexpr uint64_t kDistinctMaxPoints = 4096;      // points of a nest that are compared
 constexpr size_t kDistinctTableBytes = 48 << 10;   // constant memory for the points of all statements
 
@@ -575,8 +576,8 @@ struct Gen {
         o << in3 << "{ cl = " << e << "; key = " << make("cl") << "; }\n";
         if (A.key_idx < 0) o << in3 << "(void)key; (void)cl;\n";
         else if (repeats[a])   // (the cell tells the keys of a wide model apart, their cell field may not)
-          o << in3 << "if (cl != last" << a << ") chunk_put(a, key, cl);\n" << in3 << "last" << a << " = cl;\n";
-        else o << in3 << "chunk_put(a, key, cl);\n";
+          o << in3 << "if (cl != last" << a << ") chunk_put(a, key, cl, sweep);\n" << in3 << "last" << a << " = cl;\n";
+        else o << in3 << "chunk_put(a, key, cl, sweep);\n";
         o << in2 << "}\n";
         continue;
       }
@@ -654,10 +655,16 @@ struct Gen {
            "  unsigned long long* counts; unsigned long long lo, span; unsigned bshift, cell_shift;\n"
            "  unsigned long long* keys; const unsigned* chunk_of; const unsigned long long* c_lo;\n"
            "  const unsigned long long* c_base; const unsigned long long* c_end; unsigned long long* c_ctr;\n"
-           "  unsigned long long b0, n_buckets, low_mask; unsigned* err;\n};\n";
-      // mode 0: count keys per bucket; mode 1: route keys to their chunk's segment
-      o << "__device__ __forceinline__ void chunk_put(const ChunkJitArgs& a, unsigned long long key, "
-           "unsigned long long cell) {\n"
+           "  unsigned long long b0, n_buckets, low_mask; unsigned* err; unsigned k0, nk;\n};\n";
+      // mode 0: count keys per bucket; mode 1: route keys to their chunk's segment.
+      // A wave of at most kRouteChunks chunks is routed in two sweeps over the
+      // block's points: the first counts the block's keys per chunk (so that a
+      // block reserves once per chunk instead of every warp for every key: those
+      // atomics on a few addresses took most of the pass), the second places them.
+      o << "__shared__ unsigned sC[" << kRouteChunks << "];\n"
+           "__shared__ unsigned long long sB[" << kRouteChunks << "];\n"
+           "__device__ __forceinline__ void chunk_put(const ChunkJitArgs& a, unsigned long long key, "
+           "unsigned long long cell, int sweep) {\n"
            "  if (key == ~0ull) return;\n"
            "  const unsigned long long rel = cell - a.lo;\n"
            "  if (rel >= a.span) return;\n"
@@ -679,17 +686,21 @@ struct Gen {
            "  const unsigned k = a.chunk_of[bk];\n"
            "  if (k == 0xffffffffu) return;\n"
            "  const unsigned long long out = ((cell - a.c_lo[k]) << a.cell_shift) | (key & a.low_mask);\n"
+           "  // one reservation per chunk among the lanes here together (a warp's keys lie in\n"
+           "  // few chunks, and all warps add to the same counters)\n"
            "  const unsigned act = __activemask();\n"
-           "  const int leader = __ffs(act) - 1;\n"
-           "  const unsigned k0 = __shfl_sync(act, k, leader);\n"
-           "  unsigned long long pos;\n"
-           "  if (__all_sync(act, k == k0)) {\n"
-           "    unsigned long long base = 0;\n"
-           "    if ((int)lane == leader) base = atomicAdd(a.c_ctr + k0, (unsigned long long)__popc(act));\n"
-           "    pos = __shfl_sync(act, base, leader) + __popc(act & ((1u << lane) - 1u));\n"
-           "  } else {\n"
-           "    pos = atomicAdd(a.c_ctr + k, 1ull);\n"
+           "  const unsigned peers = __match_any_sync(act, k);\n"
+           "  const int leader = __ffs(peers) - 1;\n"
+           "  unsigned long long pos = 0;\n"
+           "  const unsigned np = __popc(peers);\n"
+           "  if (sweep == 0) {\n"
+           "    if ((int)lane == leader) atomicAdd(&sC[k - a.k0], np);\n"
+           "    return;\n"
            "  }\n"
+           "  if ((int)lane == leader)\n"
+           "    pos = sweep == 1 ? sB[k - a.k0] + atomicAdd(&sC[k - a.k0], np)\n"
+           "                     : atomicAdd(a.c_ctr + k, (unsigned long long)np);\n"
+           "  pos = __shfl_sync(peers, pos, leader) + __popc(peers & ((1u << lane) - 1u));\n"
            "  pos += a.c_base[k];\n"
            "  if (pos < a.c_end[k]) a.keys[pos] = out;\n"
            "  else atomicOr(a.err, " + std::to_string((unsigned)kErrChunkOverflow) + "u);\n"
@@ -716,6 +727,22 @@ struct Gen {
            "    __syncthreads();\n  }\n";
     }
     o << "  unsigned long long cnt = 0;\n";
+    if (chunked)
+      // sweep 0 counts, 1 places from the block's reservations, 2 places one by one (or mode 0)
+      o << "  const bool two = a.mode == 1 && a.nk != 0u;\n"
+           "  for (int sweep = two ? 0 : 2; sweep != 3; sweep = sweep == 0 ? 1 : 3) {\n"
+           "  if (two) {\n"
+           "    __syncthreads();\n"
+           "    for (unsigned k = threadIdx.x; k < a.nk; k += 128u) {\n"
+           "      if (sweep == 1) {\n"
+           "        const unsigned n = sC[k];\n"
+           "        if (n) sB[k] = atomicAdd(a.c_ctr + a.k0 + k, (unsigned long long)n);\n"
+           "      }\n"
+           "      sC[k] = 0u;\n"
+           "    }\n"
+           "    __syncthreads();\n"
+           "  }\n"
+           "  if (sweep == 1) cnt = 0;\n";
     if (!chunked)
       o << "  unsigned bi = 0;\n  for (unsigned hi = " << h.n_stmts << "u; hi - bi > 1u;) {\n"
            "    const unsigned mid = (bi + hi) >> 1;\n"
@@ -748,7 +775,7 @@ struct Gen {
     o << "    switch (" << (chunked ? "blockIdx.y" : "stmt") << ") {\n";
     for (uint32_t s = 0; s < h.n_stmts; ++s) emit_stmt(s);
     o << "    default: break;\n    }\n  }\n";
-    if (!chunked) o << "  }\n";
+    o << "  }\n";
     o << "  for (int d = 16; d > 0; d >>= 1) cnt += __shfl_xor_sync(0xffffffffu, cnt, d);\n";
     o << "  if ((threadIdx.x & 31) == 0 && cnt) atomicAdd(" << (chunked ? "a.inst" : "inst") << ", cnt);\n";
     if (!chunked)
@@ -847,6 +874,7 @@ cudaError_t jit_chunk_launch(const Model& m, const ChunkJitArgs& a, cudaStream_t
   Driver& dr = driver();
   CUfunction fn = reinterpret_cast<CUfunction>(m.jit_chunk_fn);
   ChunkJitArgs args = a;
+  if (args.nk > kRouteChunks) args.nk = 0;   // (too many for the block's counters)
   void* params[] = {&args};
   const unsigned gx = (unsigned)((m.host.n_threads + 127) / 128);
   const CUresult r = dr.launch(fn, gx, m.host.n_stmts, 1, 128, 1, 1, 0, reinterpret_cast<CUstream>(st), params, nullptr);

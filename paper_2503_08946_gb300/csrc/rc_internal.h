@@ -462,6 +462,7 @@ struct ChunkJitArgs {
   unsigned long long* c_ctr;
   uint64_t b0, n_buckets, low_mask;
   unsigned int* err;
+  uint32_t k0, nk;                    // the wave's chunks (nk = 0: none, or too many for a block's counters)
 };
 std::string jit_expand_source(const Model& m);
 std::string jit_chunk_source(const Model& m);
