@@ -399,14 +399,15 @@ rc::ScanArgs scan_args(const rc::Model& m, const rc::WorkspacePlan& p, uint8_t* 
 // unstable_first: the first pass may leave equal digits in any order (the
 // input order of a check's keys carries no meaning), so it runs as the
 // look-back-free partition pass.
+// input: the first pass reads there instead of buffer 0 (and leaves it as it is).
 rc_status enqueue_sort(const rc::WorkspacePlan& p, uint8_t* ws, uint64_t* buf0, uint64_t* buf1,
                        uint64_t spin_limit, uint32_t test_flags, cudaStream_t st, int* sorted_buf,
-                       StageTimer* tm = nullptr, bool unstable_first = false) {
+                       StageTimer* tm = nullptr, bool unstable_first = false, const uint64_t* input = nullptr) {
   uint64_t* bufs[2] = {buf0, buf1};
   auto* hist = reinterpret_cast<unsigned long long*>(ws + p.hist_off);
   auto* digoff = reinterpret_cast<unsigned long long*>(ws + p.digoff_off);
   auto* res = reinterpret_cast<rc::DevResult*>(ws + p.result_off);
-  rc_status s = cuda_status(rc::launch_digit_counts(bufs[0], p.n_keys, p.sort, hist, st));
+  rc_status s = cuda_status(rc::launch_digit_counts(input ? input : bufs[0], p.n_keys, p.sort, hist, st));
   if (s != RC_OK) return s;
   s = cuda_status(rc::launch_digit_offsets(hist, digoff, p.sort, st));
   if (s != RC_OK) return s;
@@ -415,7 +416,7 @@ rc_status enqueue_sort(const rc::WorkspacePlan& p, uint8_t* ws, uint64_t* buf0, 
   int cur = 0;
   for (uint32_t k = 0; k < p.sort.n_pass; ++k) {
     rc::SortArgs a;
-    a.keys_in = bufs[cur];
+    a.keys_in = k == 0 && input ? input : bufs[cur];
     a.keys_out = bufs[1 - cur];
     a.n = p.n_keys;
     a.shift = p.sort.shift[k];
@@ -2190,18 +2191,15 @@ rc_status rc_sort_keys(const uint64_t* keys_in, uint64_t* keys_out, uint64_t n, 
   rc::sort_clear_ranges(p.sort, n, p.hist_off, p.lookback_off, p.tilectr_off, clear);
   for (int r = 0; r < 3 && s == RC_OK; ++r) s = cuda_status(cudaMemsetAsync(ws + clear[r][0], 0, clear[r][1], st));
   if (s != RC_OK) return s;
-  // Stage the input in the output buffer and ping-pong with the workspace
-  // buffer; with an odd number of passes the result lands in the workspace
-  // buffer and is copied back.
-  s = cuda_status(cudaMemcpyAsync(keys_out, keys_in, n * 8, cudaMemcpyDeviceToDevice, st));
-  if (s != RC_OK) return s;
+  // The first pass reads the input where it is; the passes then alternate between
+  // the output and the workspace buffer, such that the last one ends in the output.
+  if (p.sort.n_pass == 0) return cuda_status(cudaMemcpyAsync(keys_out, keys_in, n * 8, cudaMemcpyDeviceToDevice, st));
+  uint64_t* bufs[2] = {keys_out, reinterpret_cast<uint64_t*>(ws + pong)};
+  if (p.sort.n_pass & 1u) std::swap(bufs[0], bufs[1]);
   int sorted = 0;
   const bool stall = rc::sort_stall_requested();
-  s = enqueue_sort(p, ws, keys_out, reinterpret_cast<uint64_t*>(ws + pong), stall ? 4096ull : (1ull << 20),
-                   stall ? (uint32_t)RC_TEST_STALL_LOOKBACK : 0u, st, &sorted);
-  if (s != RC_OK) return s;
-  if (sorted == 1) s = cuda_status(cudaMemcpyAsync(keys_out, ws + pong, n * 8, cudaMemcpyDeviceToDevice, st));
-  return s;
+  return enqueue_sort(p, ws, bufs[0], bufs[1], stall ? 4096ull : (1ull << 20),
+                      stall ? (uint32_t)RC_TEST_STALL_LOOKBACK : 0u, st, &sorted, nullptr, false, keys_in);
 }
 
 rc_status rc_sort_status(const void* workspace, void* stream) {

@@ -86,15 +86,21 @@ extern "C" rc_status rc_sort_keys_static(const uint64_t* keys_in, uint64_t* keys
   size_t clear[3][2];
   rc::sort_clear_ranges(sp, n, kOffHist, kOffLookback, kOffTileCtr, clear);
   for (int r = 0; r < 3 && st == RC_OK; ++r) st = as_status(cudaMemsetAsync(s + clear[r][0], 0, clear[r][1], cs));
-  if (st == RC_OK) st = as_status(cudaMemcpyAsync(keys_out, keys_in, n * 8, cudaMemcpyDeviceToDevice, cs));
-  if (st == RC_OK) st = as_status(rc::launch_digit_counts(keys_out, n, sp, hist, cs));
+  if (sp.n_pass == 0 && st == RC_OK)
+    return as_status(cudaMemcpyAsync(keys_out, keys_in, n * 8, cudaMemcpyDeviceToDevice, cs));
+  if (st == RC_OK) st = as_status(rc::launch_digit_counts(keys_in, n, sp, hist, cs));
   if (st == RC_OK) st = as_status(rc::launch_digit_offsets(hist, digoff, sp, cs));
+  // (the first pass reads the input, the last one ends in the output)
   uint64_t* bufs[2] = {keys_out, pong};
+  if (sp.n_pass & 1u) {
+    bufs[0] = pong;
+    bufs[1] = keys_out;
+  }
   const bool stall = rc::sort_stall_requested();
   int cur = 0;
   for (uint32_t k = 0; k < sp.n_pass && st == RC_OK; ++k) {
     rc::SortArgs a;
-    a.keys_in = bufs[cur];
+    a.keys_in = k == 0 ? keys_in : bufs[cur];
     a.keys_out = bufs[1 - cur];
     a.n = n;
     a.shift = sp.shift[k];
@@ -110,6 +116,5 @@ extern "C" rc_status rc_sort_keys_static(const uint64_t* keys_in, uint64_t* keys
     st = as_status(rc::launch_onesweep(a, rc::radix_bits_for(a.bits), cs));
     cur = 1 - cur;
   }
-  if (st == RC_OK && cur == 1) st = as_status(cudaMemcpyAsync(keys_out, pong, n * 8, cudaMemcpyDeviceToDevice, cs));
   return st;
 }
