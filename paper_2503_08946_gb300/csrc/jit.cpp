@@ -517,6 +517,12 @@ struct Gen {
       o << in2 << "const " << row_type(S.row_phase) << " ph = " << row(S.row_phase) << ";\n";
     }
     o << in2 << "(void)ph;\n";
+    // Statements with thread-dependent trips: every thread writes its own run, so
+    // each 8-byte store of a warp is 32 sectors; the keys of a point are stored in
+    // pairs where the run is 16-byte aligned.
+    const bool pairs = !chunked && !S.dense && S.n_key > 1;
+    if (pairs)
+      for (int kq = 0; kq < S.n_key; ++kq) o << in2 << "unsigned long long k" << kq << " = ~0ull;\n";
     const bool cl32 = m.total_cells < (1ull << 32);
     for (int a = 0; a < S.n_acc; ++a) {
       const DevAccess& A = accs[S.acc0 + a];
@@ -600,6 +606,7 @@ struct Gen {
                 : "(unsigned)(((cl * " + ulit(kCellHashMul) + ") & hmask) >> hsh)")
         << "], 1u);\n" << in3 << "}\n";
       if (S.dense) o << in3 << "out[" << ulit((uint64_t)A.key_idx * T) << "] = key;\n";
+      else if (pairs) o << in3 << "k" << A.key_idx << " = key;\n";
       else o << in3 << "out[" << A.key_idx << "] = key;\n";
       o << in2 << "}\n";
     }
@@ -607,6 +614,15 @@ struct Gen {
     else
       o << in2 << "cnt += " << S.n_acc << "u * (" << (chunked ? "" : "all_points ? 1u : ") << "(unsigned)pts" << s
         << "[p].y);\n";
+    if (pairs) {
+      o << in2 << "if (((unsigned long long)out & 15ull) == 0ull) {\n";
+      for (int kq = 0; kq + 1 < S.n_key; kq += 2)
+        o << in2 << "  *reinterpret_cast<ulonglong2*>(out + " << kq << ") = make_ulonglong2(k" << kq << ", k" << kq + 1 << ");\n";
+      if (S.n_key & 1) o << in2 << "  out[" << S.n_key - 1 << "] = k" << S.n_key - 1 << ";\n";
+      o << in2 << "} else {\n";
+      for (int kq = 0; kq < S.n_key; ++kq) o << in2 << "  out[" << kq << "] = k" << kq << ";\n";
+      o << in2 << "}\n";
+    }
     if (!S.dense && !chunked) o << in2 << "out += " << S.n_key << ";\n";
     o << ind << "}";
     if (chunked) {
