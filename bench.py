@@ -1,7 +1,7 @@
 #!/usr/bin/env python
 """Benchmark of the concrete-instance race check on GB300.
 
-One step = one full check (expansion, onesweep sort, segmented scan, witness)
+One step = one full check (expansion, two partition passes, cell test, witness)
 of the seeded random affine kernel model: 4096 blocks x 256 threads, 36
 statements with loop nests of depth <= 2 and trip counts 1-16, 4 arrays in a
 2^30-cell space, 8 barrier intervals, ~1.1e9 access instances (seed 0).  The
@@ -59,14 +59,15 @@ def load_peaks():
 
 
 KERNEL_SOURCES = {"onesweep": "sort.cu", "partition": "sort.cu", "partition_a": "bucket.cu",
-                  "partition_b": "bucket.cu", "local_sort": "bucket.cu", "histogram_b": "bucket.cu",
+                  "partition_b": "bucket.cu", "cell_test": "filter.cu", "histogram_b": "bucket.cu",
                   "scan": "scan.cu", "expand": "jit.cpp", "histogram": "bucket.cu"}
 
 
 # the part of a source file that holds a kernel and its helpers (first line
 # starting with the first marker up to the line starting with the second); a
 # kernel without an entry is hashed with its whole file
-KERNEL_REGIONS = {"local_sort": ("// Exclusive scan in place of n counters", "// one thread per result: the bucket")}
+KERNEL_REGIONS = {"partition_a": ("// partition passes (unstable", "// pass-B histogram: keys per"),
+                  "partition_b": ("// partition passes (unstable", "// pass-B histogram: keys per")}
 
 
 def kernel_source_hash(kernel="onesweep"):
@@ -293,13 +294,15 @@ def run_native(args):
     }
     peak, peak_kind = load_peaks()
     # per kernel: (algorithmic bytes per launch, mean launch ms).  Every pass
-    # (partition, local sort, radix pass) reads and writes each key once (16 B
-    # per key); expansion writes 8 B, histograms and the scan read 8 B.
+    # (partition, radix pass) reads and writes each key once (16 B per key);
+    # expansion writes 8 B, histograms, the cell test and the scan read 8 B.
     if bucketed:
-        names = {3: ["partition_a", "partition_b", "local_sort"], 2: ["partition_a", "local_sort"],
-                 1: ["local_sort"]}[n_pass]
-        kern = {nm: (16.0 * n_keys, st_mean["sort_pass_ms"][i]) for i, nm in enumerate(names)}
-        kern["histogram_b"] = (8.0 * n_keys, st_mean["histogram2_ms"])
+        names = {3: ["partition_a", "partition_b", "cell_test"], 2: ["partition_a", "cell_test"],
+                 1: ["cell_test"]}[n_pass]
+        kern = {nm: ((8.0 if nm == "cell_test" else 16.0) * n_keys, st_mean["sort_pass_ms"][i])
+                for i, nm in enumerate(names)}
+        if n_pass == 3:
+            kern["histogram_b"] = (8.0 * n_keys, st_mean["histogram2_ms"])
     else:
         kern = {"onesweep": (16.0 * n_keys, mean(st_mean["sort_pass_ms"][1:] or st_mean["sort_pass_ms"]))}
         if n_pass:
@@ -308,7 +311,8 @@ def run_native(args):
     hist_fused = bool(stages[0].get("histogram_fused"))
     if not hist_fused:   # (else the expansion counted it: no pass over the keys)
         kern["histogram"] = (8.0 * n_keys, st_mean["histogram_ms"])
-    kern["scan"] = (8.0 * n_keys, st_mean["scan_ms"])
+    if not bucketed:   # (the cell test has no scan)
+        kern["scan"] = (8.0 * n_keys, st_mean["scan_ms"])
     launches = {"onesweep": max(1, n_pass - 1)} if not bucketed else {}
     dominant = max(kern, key=lambda k: kern[k][1] * launches.get(k, 1))
     alg_bytes, dur_ms = kern[dominant]
@@ -321,8 +325,8 @@ def run_native(args):
     per_kernel = {k: {"ms": v[1], "alg_bytes_per_key": v[0] / n_keys,
                       "frac": v[0] / (v[1] / 1e3) / 1e9 / peak if v[1] > 0 else None} for k, v in kern.items()}
     # the whole check: expansion 8, histograms 8 each (none for a histogram the
-    # expansion counts), passes 16 each, scan 8 bytes per key
-    pk = 8 + (0 if hist_fused else 8) + 16 * n_pass + 8 + (8 if bucketed and n_pass == 3 else 0)
+    # expansion counts), passes 16 each, cell test or scan 8 bytes per key
+    pk = 8 + (0 if hist_fused else 8) + 8 + (16 * (n_pass - 1) + (8 if n_pass == 3 else 0) if bucketed else 16 * n_pass)
     pipeline_bytes = pk * n_keys
     pipeline = {"alg_bytes_per_key": pk,
                 "gbs": pipeline_bytes / (st_mean["check_ms"] / 1e3) / 1e9,
@@ -383,16 +387,16 @@ def run_native(args):
             "scaling": "weak", "vs_baseline": None, "dtype": "u64", "data": "synthetic",
             "config": {"workload": WORKLOAD if args.blocks == 4096 else WORKLOAD.replace("4096 blocks", f"{args.blocks} blocks"),
                        "seed": args.seed, "instances_per_rank": instances,
-                       "keys": n_keys, "sort_bits": lay["sort_hi"] - lay["sort_lo"], "sort_passes": n_pass,
-                       "path": "bucket" if bucketed else "lsd sort", "l2": "inputs larger than L2 (key buffers ~9 GB)",
+                       "keys": n_keys, "keys_of": "one per distinct point of a loop nest (every point is counted in instances)", "sort_bits": lay["sort_hi"] - lay["sort_lo"], "sort_passes": n_pass,
+                       "path": "bucket" if bucketed else "lsd sort", "l2": "inputs larger than L2 (key buffers of several GB)",
                        "parallelism": f"independent models per rank x{world}"},
             "result": result,
             "roofline": roofline, "pipeline": pipeline, "stages_ms": st_mean,
             "cpu_baseline": cpu, "e2e": e2e, "clocks": clocks,
-            # our kernels per check: bucket path 20 with two partition passes (init, expansion,
-            # 2 x (histogram, offsets), 2 passes, local sort, tail, scan (3), finish, witness (4);
-            # offsets of pass B: 3); LSD path 11 + passes
-            "gpu_launches": (({3: 19, 2: 14, 1: 12}[n_pass] - (1 if hist_fused else 0)) if bucketed else (11 + n_pass)) * args.steps,
+            # our kernels per check: bucket path 14 with two partition passes (start, expansion,
+            # 2 x (histogram, offsets), 2 passes, cell test, finish, witness (4)); LSD path 11 + passes
+            "gpu_launches": (({3: 14, 2: 11, 1: 9}[n_pass] - (1 if hist_fused and n_pass > 1 else 0)) if bucketed
+                             else (11 + n_pass)) * args.steps,
         }
         line.update(subs)
         print(json.dumps(line), flush=True)

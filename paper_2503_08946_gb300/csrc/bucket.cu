@@ -246,7 +246,7 @@ constexpr size_t bpart_smem() {
 // keys), so a tile is read from it once and its keys stay in registers until the
 // scatter, with digit and rank in one word (recomputing the digit spilled and took
 // 8 % longer); destinations are 32-bit (a bucketed buffer has fewer than 2^32 keys) and
-// a key with bit 63 is padding.  290 M keys of the 4096 x 256 random affine model:
+// a key with bit 63 is padding.  303 M keys of the 4096 x 256 random affine model:
 // 9-bit pass A 1.06 ms (1.17 with one 64-bit claim per digit), 8-bit pass B
 // 1.01 ms (1.07).  Loading the tile straight into registers was slower (pass B
 // 1.25 ms: the loads in flight need L1 lines), as were 3 and 5 blocks per SM.

@@ -34,14 +34,15 @@
 //
 // What bounds it: one read of every key (8 bytes); about 78 warp instructions per
 // 32 keys keep the issue slots 76 % busy.  On the 4096 x 256 random affine model
-// (578 M keys, 2^17 buckets of 4,400 keys) 1.35 ms, where the counting sort of
-// every bucket and the cell scan that it replaces there took 3.52 + 1.66 ms; on
-// 49 M keys with hot cells 0.26 ms against 1.63 + 0.22 ms.  Blocks of 256 threads
-// with 20 keys each in registers, 4 per SM, were the fastest split without spills
-// (512 threads, 2 per SM: 1.95 ms; 384 threads with 16 keys, 3 per SM: 1.51 ms):
-// the barriers between the steps stall fewer warps.  The hashed table (HT) takes
-// 3 blocks per SM; on 2,000 small models in one batch (34 cell bits, 18 million
-// kept keys) the check takes 1.99 ms with it, 2.62 ms with the local sort and scan.
+// with a key per point (578 M keys, 2^17 buckets of 4,400 keys) 1.35 ms, where the
+// counting sort of every bucket and the cell scan that it replaces there took
+// 3.52 + 1.66 ms; on 49 M keys with hot cells 0.26 ms against 1.63 + 0.22 ms.  (With
+// a key per distinct point: 303 M keys in 0.94 ms.)  Blocks of 256 threads with 20
+// keys each in registers, 4 per SM, were the fastest split without spills (512
+// threads, 2 per SM: 1.95 ms; 384 threads with 16 keys, 3 per SM: 1.51 ms): the
+// barriers between the steps stall fewer warps.  The hashed table (HT) takes 3
+// blocks per SM; on 2,000 small models in one batch (34 cell bits, some 28 M kept
+// keys) the check takes 1.99 ms with it, 2.62 ms with the local sort and scan.
 #include <cuda_runtime.h>
 
 #include "fold.cuh"
