@@ -130,6 +130,7 @@ struct DistinctPoints {
 };
 constexpr unsigned kRouteChunks = 1024;            // chunks of a wave routed in two sweeps
 constexpr uint64_t kDistinctMaxPoints = 4096;      // points of a nest that are compared
+constexpr size_t kConstantBytes = 60 << 10;
 constexpr size_t kDistinctTableBytes = 48 << 10;   // constant memory for the points of all statements
 
 struct Gen {
@@ -223,7 +224,11 @@ struct Gen {
     const uint32_t ns = m.host.n_stmts;
     dp.resize(ns);
     check_base.assign(ns, 0);
-    size_t budget = kDistinctTableBytes;
+    // (constant memory holds 64 KB, of which the block table takes 12 bytes a statement)
+    const size_t blk_bytes = 12 * ((size_t)ns + 1);
+    size_t budget = blk_bytes + kDistinctTableBytes <= kConstantBytes ? kDistinctTableBytes
+                    : blk_bytes < kConstantBytes                      ? kConstantBytes - blk_bytes
+                                                                      : 0;
     for (uint32_t s = 0; s < ns; ++s) {
       const DevStmt& S = stmts[s];
       if (!S.dense) continue;
