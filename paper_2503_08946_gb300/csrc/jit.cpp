@@ -468,7 +468,7 @@ struct Gen {
       bool fixed = fixed_inside(S, S.row_phase) && (S.row_wphase < 0 || fixed_inside(S, S.row_wphase));
       for (int d = 0; d < A.ndims; ++d) fixed = fixed && fixed_inside(S, A.row0 + d);
       repeats[a] = fixed;
-      if (fixed) o << "      unsigned long long last" << a << " = ~0ull;\n";
+      if (fixed) o << "      unsigned long long last" << a << " = ~0ull" << (chunked ? ", lastc" + std::to_string(a) + " = ~0ull" : std::string()) << ";\n";
     }
     emit_terms(S, 0, "      ");
     std::string ind = "      ";
@@ -586,8 +586,11 @@ struct Gen {
         if (!sure) o << in3 << "if (dc != 0xFFFFFFFFu) " << report << "\n" << in3 << "else\n";
         o << in3 << "{ cl = " << e << "; key = " << make("cl") << "; }\n";
         if (A.key_idx < 0) o << in3 << "(void)key; (void)cl;\n";
-        else if (repeats[a])   // (the cell tells the keys of a wide model apart, their cell field may not)
-          o << in3 << "if (cl != last" << a << ") chunk_put(a, key, cl, sweep);\n" << in3 << "last" << a << " = cl;\n";
+        else if (repeats[a])
+          // the same instance again: the same cell (a wide model's key may not hold all of it)
+          // and the same fields below it, the interval among them, which an outer loop may move
+          o << in3 << "if (cl != lastc" << a << " || key != last" << a << ") chunk_put(a, key, cl, sweep);\n"
+            << in3 << "lastc" << a << " = cl;\n" << in3 << "last" << a << " = key;\n";
         else o << in3 << "chunk_put(a, key, cl, sweep);\n";
         o << in2 << "}\n";
         continue;
