@@ -480,11 +480,13 @@ struct Gen {
       o << ind << "unsigned e = " << (chunked ? "" : "all_points ? p : ") << "(unsigned)pts" << s << "[p].x;\n";
       for (int l = S.n_loops - 1; l >= 0; --l) {
         const std::string k = "(e" + (l ? " % " + std::to_string(S.trips[l]) + "u" : std::string()) + ")";
+        // (the iterator fits its type, the step times the point's number may not: it wraps)
         if (n_it[l])
-          o << ind << "const int i" << l << " = " << row32(S.row_lower[l]) << " + " << S.step[l] << " * (int)" << k << ";\n";
+          o << ind << "const int i" << l << " = (int)((unsigned)" << row32(S.row_lower[l]) << " + " << S.step[l]
+            << "u * (unsigned)" << k << ");\n";
         else
-          o << ind << "const long long i" << l << " = " << row64(S.row_lower[l]) << " + " << lit(S.step[l])
-            << " * (long long)" << k << ";\n";
+          o << ind << "const long long i" << l << " = (long long)((unsigned long long)" << row64(S.row_lower[l]) << " + "
+            << ulit((uint64_t)S.step[l]) << " * (unsigned long long)" << k << ");\n";
         if (l) o << ind << "e /= " << S.trips[l] << "u;\n";
       }
       for (int l = 0; l < S.n_loops; ++l) emit_terms(S, l + 1, ind);
