@@ -212,6 +212,96 @@ struct Gen {
     }
   }
 
+  // Whether every point differs from all others in some row, shown without looking
+  // at the points: a row whose coefficients grow faster than what the smaller ones
+  // can add up to tells the numbers of its loops (a mixed radix), and what is known
+  // leaves the other rows with fewer loops.  (False: not shown.)
+  static bool all_points_differ(const DevStmt& S, const std::vector<std::vector<uint64_t>>& co) {
+    uint32_t known = 0;
+    for (int l = 0; l < S.n_loops; ++l)
+      if (S.trips[l] <= 1) known |= 1u << l;
+    for (bool more = true; more;) {
+      more = false;
+      for (const std::vector<uint64_t>& c : co) {
+        std::vector<std::pair<unsigned __int128, int>> a;   // (magnitude, loop)
+        for (int l = 0; l < S.n_loops; ++l) {
+          const int64_t v = (int64_t)c[l];
+          if (v != 0 && !((known >> l) & 1u)) a.emplace_back(v < 0 ? -(__int128)v : (__int128)v, l);
+        }
+        if (a.empty()) continue;
+        std::sort(a.begin(), a.end());
+        unsigned __int128 sum = 0;   // (trips are at most kDistinctMaxPoints)
+        bool radix = true;
+        for (const auto& x : a) {
+          radix = radix && x.first > sum;
+          sum += x.first * (unsigned __int128)(S.trips[x.second] - 1);
+        }
+        if (!radix || sum >> 63) continue;   // (rows are evaluated modulo 2^64)
+        for (const auto& x : a) known |= 1u << x.second;
+        more = true;
+      }
+    }
+    return known == (1u << S.n_loops) - 1u;
+  }
+
+  // The distinct points in order of their first, if they are at most `most`: the
+  // loops that move some row are run through, the others multiply.
+  bool enumerate_points(const DevStmt& S, const std::vector<std::vector<uint64_t>>& co, size_t most, DistinctPoints* p) {
+    const size_t nr = co.size();
+    std::vector<int> moving;
+    std::vector<uint64_t> stride(S.n_loops);
+    uint64_t n = 1, times = 1, at = 1;
+    for (int l = S.n_loops - 1; l >= 0; --l) {
+      stride[l] = at;
+      at *= (uint64_t)S.trips[l];
+      bool moves = false;
+      for (size_t r = 0; r < nr; ++r) moves = moves || co[r][l] != 0;
+      if (moves) {
+        moving.insert(moving.begin(), l);
+        n *= (uint64_t)S.trips[l];
+      } else {
+        times *= (uint64_t)S.trips[l];
+      }
+    }
+    // an open-addressed table of the points found (1 + their number) and their images
+    size_t cap = 64;
+    while (cap < 2 * n) cap *= 2;
+    point_table.assign(cap, 0u);
+    point_images.clear();
+    std::vector<uint64_t> im(nr, 0);
+    std::vector<int64_t> k(moving.size(), 0);
+    uint64_t e = 0;
+    for (uint64_t x = 0; x < n; ++x) {
+      uint64_t h = 0;
+      for (uint64_t v : im) h = (h ^ v) * 0x9E3779B97F4A7C15ull, h ^= h >> 29;
+      size_t i = (size_t)h & (cap - 1);
+      for (; point_table[i] != 0u; i = (i + 1) & (cap - 1))
+        if (std::equal(im.begin(), im.end(), point_images.begin() + (size_t)(point_table[i] - 1u) * nr)) break;
+      if (point_table[i] == 0u) {
+        if (p->point.size() >= most) return false;
+        p->point.push_back((uint32_t)e);
+        p->times.push_back(0);
+        point_images.insert(point_images.end(), im.begin(), im.end());
+        point_table[i] = (uint32_t)p->point.size();
+      }
+      p->times[point_table[i] - 1u] += (uint32_t)times;
+      for (size_t q = moving.size(); q-- > 0;) {   // the next point
+        const int l = moving[q];
+        if (++k[q] < S.trips[l]) {
+          e += stride[l];
+          for (size_t r = 0; r < nr; ++r) im[r] += co[r][l];
+          break;
+        }
+        k[q] = 0;
+        e -= stride[l] * (uint64_t)(S.trips[l] - 1);
+        for (size_t r = 0; r < nr; ++r) im[r] -= co[r][l] * (uint64_t)(S.trips[l] - 1);
+      }
+    }
+    return true;
+  }
+  std::vector<uint32_t> point_table;   // scratch of enumerate_points
+  std::vector<uint64_t> point_images;
+
   // The points of a dense statement's loop nest that differ in some row.  A
   // point enters an instance only through the rows of the statement (guards,
   // intervals, indices, operands of its terms), each linear in the iterators, so
@@ -257,28 +347,11 @@ struct Gen {
           for (uint64_t v : c) zero = zero && v == 0;
           if (!zero && std::find(co.begin(), co.end(), c) == co.end()) co.push_back(c);
         }
-        std::map<std::vector<uint64_t>, uint32_t> seen;
         DistinctPoints p;
-        std::vector<uint64_t> im(co.size());
-        for (uint32_t e = 0; e < S.n_iter; ++e) {
-          std::fill(im.begin(), im.end(), 0);
-          uint64_t rest = e;
-          for (int l = S.n_loops - 1; l >= 0; --l) {
-            const uint64_t k = rest % (uint64_t)S.trips[l];
-            rest /= (uint64_t)S.trips[l];
-            for (size_t r = 0; r < co.size(); ++r) im[r] += co[r][l] * k;
-          }
-          const auto it = seen.emplace(im, (uint32_t)p.point.size());
-          if (it.second) {
-            p.point.push_back(e);
-            p.times.push_back(0);
-          }
-          ++p.times[it.first->second];
-        }
         // (a table and a division per point: worth it from a tenth of the points on)
-        const size_t bytes = 4 * p.point.size();
-        if (p.point.size() * 10 <= S.n_iter * 9 && bytes <= budget) {
-          budget -= bytes;
+        const size_t most = std::min<size_t>(budget / 4, (size_t)(S.n_iter * 9 / 10));
+        if (!all_points_differ(S, co) && enumerate_points(S, co, most, &p)) {
+          budget -= 4 * p.point.size();
           n_pts = p.point.size();
           dp[s] = std::move(p);
         }
