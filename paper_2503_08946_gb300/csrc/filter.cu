@@ -74,19 +74,23 @@ constexpr uint64_t hash_inverse() {
 }
 static_assert(hash_inverse() * kCellHashMul == 1ull, "inverse of the cell hash multiplier");
 
-// Slots of a table.  Direct (r <= kFilterMaxSlotBits): the slot is the cell's r
-// hash bits, and the table has room for at least 256 candidate cells of 16
-// intervals each.  Hashed (HT, larger r): 2^kFilterMaxSlotBits slots with a tag.
-__host__ __device__ __forceinline__ unsigned table_words(uint32_t r) {
-  return r < 12 ? 4096u : r > kFilterMaxSlotBits ? 1u << kFilterMaxSlotBits : 1u << r;
+// Words of a table.  Direct (r <= kFilterMaxSlotBits): the slot is the cell's r
+// hash bits.  At least 4096, and up to 2^kFilterMaxSlotBits where every cell's
+// intervals (two 16-bit entries of step 3 a word) would fill them: with half as many
+// a tile buffer of 42 M keys in one-pass buckets took 0.38 ms instead of 0.33.
+// Hashed (HT, larger r): 2^kFilterMaxSlotBits slots with a tag.
+unsigned table_words(uint32_t r, uint32_t phase_bits) {
+  const uint32_t bits = r + phase_bits > 13u ? r + phase_bits - 1u : 12u;
+  return 1u << (bits > kFilterMaxSlotBits || r > kFilterMaxSlotBits ? kFilterMaxSlotBits : bits > r ? bits : r);
 }
 __host__ __device__ __forceinline__ unsigned mask_words(uint32_t r) {
   return r < 5 ? 1u : r > kFilterMaxSlotBits ? 1u << (kFilterMaxSlotBits - 5) : 1u << (r - 5);
 }
 // (four words behind the table: the slot of padding keys and of cells without a write)
-size_t filter_smem(uint32_t r, bool at) {
-  const size_t tw = table_words(r), mw = mask_words(r);
-  return (tw + 4 + (r > kFilterMaxSlotBits ? tw : 0) + (at ? 10 : 5) * mw + 1 + (at ? 3 * tw / 32 : 0)) * sizeof(unsigned);
+size_t filter_smem(uint32_t r, uint32_t phase_bits, bool at) {
+  const size_t tw = table_words(r, phase_bits), mw = mask_words(r);
+  return (tw + 4 + (r > kFilterMaxSlotBits ? tw : 0) + (at ? 10 : 5) * mw + 1 + (at ? 3 * (2 * tw / 32) : 0)) *
+         sizeof(unsigned);
 }
 
 // One block per bucket.  A bucket of at most kFltCap keys is held in registers
@@ -103,7 +107,7 @@ size_t filter_smem(uint32_t r, bool at) {
 template <bool PAD, bool REGS, bool AT, bool HT>
 __device__ __forceinline__ void filter_bucket(const FilterArgs& a, const uint64_t* src, uint64_t len) {
   extern __shared__ __align__(16) unsigned s_tab[];
-  const unsigned tw = table_words(a.r), mw = mask_words(a.r);
+  const unsigned tw = a.tw, mw = mask_words(a.r);
   unsigned* s_tag = s_tab + tw + 4;     // (HT) the cell of every slot
   unsigned* s_two = s_tag + (HT ? tw : 0u);   // cells with two threads of a block, a bit per slot
   unsigned* s_wi = s_two + mw;          // cells with writes in two intervals, then the candidate cells
@@ -118,8 +122,8 @@ __device__ __forceinline__ void filter_bucket(const FilterArgs& a, const uint64_
   unsigned* s_wp = s_r + mw;
   unsigned* s_rp = s_wp + mw;
   unsigned* s_e2 = s_rp + mw;
-  unsigned* s_ew = s_e2 + tw / 32;
-  unsigned* s_er = s_ew + tw / 32;
+  unsigned* s_ew = s_e2 + 2 * tw / 32;
+  unsigned* s_er = s_ew + 2 * tw / 32;
   __shared__ unsigned s_wsum[kFltThreads / 32];
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
   const uint32_t pb = a.s.phase_bits, bb = a.s.block_bits, tb = a.s.thread_bits;
@@ -319,30 +323,42 @@ __device__ __forceinline__ void filter_bucket(const FilterArgs& a, const uint64_
       if (!((m >> (s & 31u)) & 1u)) return ~0u;
       return ((s_rank[s >> 5] + __popc(m & ((1u << (s & 31u)) - 1u))) << pb) | (unsigned)((uint64_t)k >> (kb + bb + tb));
     };
-    // windows of tw entries of the table
-    for (unsigned e0 = 0; e0 < (ncand << pb); e0 += tw) {
-      const unsigned used = min(tw, (ncand << pb) - e0);
-      clear_table((used + 3u) & ~3u);
+    // Windows of the table; the bucket is read twice for each.  All keys of a candidate
+    // lie in one block (a key of another block has decided its cell), so where a larger
+    // bucket is read from memory an entry holds the thread of a write alone, in 16 bits
+    // if it fits: half as many windows.  (A bucket in registers costs no reads.)
+    const bool half = !REGS && tb <= kFilterHalfThreadBits;
+    unsigned short* s_tab16 = reinterpret_cast<unsigned short*>(s_tab);
+    const unsigned tmask = (1u << tb) - 1u;   // (a block has at most 2^20 threads)
+    auto thread_of = [&](unsigned k) { return (((k >> kb) & tmask) << 1) | 1u; };
+    const unsigned room = half ? 2u * tw : tw;
+    for (unsigned e0 = 0; e0 < (ncand << pb); e0 += room) {
+      const unsigned used = min(room, (ncand << pb) - e0);
+      clear_table(((half ? (used + 1u) / 2u : used) + 3u) & ~3u);
       if constexpr (AT)
-        for (unsigned i = tid; i < 3 * (tw / 32); i += kFltThreads) s_e2[i] = 0;
+        for (unsigned i = tid; i < 3 * (2 * tw / 32); i += kFltThreads) s_e2[i] = 0;
       __syncthreads();
       each([&](unsigned k, unsigned s) {
         if (k & kmask) {
           const unsigned e = entry(k, s) - e0;
-          if (e < used) s_tab[e] = k;
+          if (e < used) {
+            if (half) s_tab16[e] = (unsigned short)thread_of(k);
+            else s_tab[e] = k;
+          }
         }
       });
       __syncthreads();
       each([&](unsigned k, unsigned s) {
         const unsigned e = entry(k, s) - e0;
         if (e < used) {
-          const unsigned rep = s_tab[e];
+          const unsigned rep = half ? s_tab16[e] : s_tab[e];
+          const bool other = half ? rep != thread_of(k) : ((rep ^ k) & m_bt) != 0u;
           if constexpr (AT) {
             if (rep == 0u) return;
-            if ((rep ^ k) & m_bt) mark(s_e2, e);
+            if (other) mark(s_e2, e);
             if ((k & kmask) != 2u) mark(k & kmask ? s_ew : s_er, e);
           } else {
-            if (rep != 0u && ((rep ^ k) & m_bt) != 0u) mark(s_hot, (e + e0) >> pb);
+            if (rep != 0u && other) mark(s_hot, (e + e0) >> pb);
           }
         }
       });
@@ -426,9 +442,9 @@ __global__ void __launch_bounds__(kFltThreads, HT ? 3 : kFltBlocks) bucket_filte
 template <bool PAD, bool AT, bool HT>
 cudaError_t launch_filter(const FilterArgs& a, uint32_t D, cudaStream_t st) {
   const cudaError_t e = ensure_kernel_smem(reinterpret_cast<const void*>(bucket_filter_kernel<PAD, AT, HT>),
-                                           filter_smem(HT ? 31 : kFilterMaxSlotBits, AT));
+                                           filter_smem(HT ? 31 : kFilterMaxSlotBits, 0, AT));
   if (e != cudaSuccess) return e;
-  bucket_filter_kernel<PAD, AT, HT><<<1u << D, kFltThreads, filter_smem(a.r, AT), st>>>(a);
+  bucket_filter_kernel<PAD, AT, HT><<<1u << D, kFltThreads, filter_smem(a.r, a.s.phase_bits, AT), st>>>(a);
   return cudaGetLastError();
 }
 template <bool PAD>
@@ -441,7 +457,9 @@ cudaError_t launch_filter(const FilterArgs& a, uint32_t D, cudaStream_t st) {
 
 }  // namespace
 
-cudaError_t launch_bucket_filter(const FilterArgs& a, uint32_t D, cudaStream_t st) {
+cudaError_t launch_bucket_filter(const FilterArgs& args, uint32_t D, cudaStream_t st) {
+  FilterArgs a = args;
+  a.tw = table_words(a.r, a.s.phase_bits);
   if (a.r > kFilterMaxTagBits || a.s.cell_shift > kFilterMaxLowBits) return cudaErrorInvalidValue;
   // an unpartitioned bucket holds padding keys, which take the word behind the table
   return D == 0 ? launch_filter<true>(a, D, st) : launch_filter<false>(a, D, st);

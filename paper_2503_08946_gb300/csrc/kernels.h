@@ -253,6 +253,7 @@ struct FilterArgs {
   const uint64_t* keys_in;
   const unsigned long long* boff;
   uint32_t r;                       // hash bits below the bucket bits = slot bits (tag bits above kFilterMaxSlotBits)
+  uint32_t tw;                      // words of a table (set by the launcher)
   uint64_t hmask;                   // 2^(cell bits) - 1 of the whole hash
   uint64_t part_hash;               // a hash part's top bits of the hash, 0 for a whole check
 };

@@ -349,17 +349,32 @@ constexpr int kPartTileHost = kSortThreadsHost * 16;    // keys per tile of the 
 // inside its block's registers (5,120) with room for the spread; 6,000 and 9,000
 // keys with larger blocks measured slower.  A slot per cell needs cell bits -
 // kFilterMaxSlotBits bucket bits; where that makes buckets of fewer than
-// kFilterMinKeys keys (mostly empty tables), the tables are hashed.  One partition
-// pass of 10 bits and larger buckets, read again from L2, where that suffices:
-// Ge-SpMM with 54 M key slots 0.76 ms in one pass, 0.92 ms in two.
+// kFilterMinKeys keys (mostly empty tables), the tables are hashed.
+//
+// One partition pass of 10 bits and larger buckets, read again in every step, against
+// two passes and buckets in registers: a bucket is read twice, and twice more for
+// every table of candidates (a candidate's intervals take an entry each), where the
+// second pass and its histogram move 24 bytes a key.  So the line is the number of
+// tables if every cell were a candidate: two.  Checks in one and in two passes, ms,
+// at 5 to 67 M slots (up to 64 K a bucket):
+//   no second interval, or two (histograms)          0.15 / 0.19, 0.44 / 0.56, 0.82 / 1.05
+//   every cell a candidate (tile buffers), 1 table   0.19 / 0.21, 0.33 / 0.34
+//                                          2 tables  0.75 / 0.65, 0.78 / 0.64
+//                                          4 tables  2.0 / 1.2
+//   few candidates (Ge-SpMM), at most 1, 2, 4 tables 0.46 / 0.53, 0.80 / 0.96, 0.73 / 0.86
+// Larger buckets were measured with Ge-SpMM only (109 M slots 1.6 / 1.9, 213 M 3.3 /
+// 3.9): the line of 64 K slots a bucket is the largest size seen with all three.
 constexpr uint32_t kFilterMaxSlotBits = 13;         // table slots of a bucket: 32 KB of 4-byte words
 constexpr uint32_t kFilterMaxTagBits = 31;          // hash bits below the bucket bits, with a hashed table
 constexpr uint32_t kFilterMaxLowBits = 32;          // (interval, block, thread, kind) bits: a table word
 constexpr uint64_t kFilterTarget = 4600;            // planned mean keys per bucket (at most)
 constexpr uint64_t kFilterMinKeys = 512;            // ... and at least, where the cell bits ask for more buckets
-constexpr uint32_t kFilterMaxPhaseBits = 6;         // intervals: a bucket's candidates take a dozen tables at most
+constexpr uint32_t kFilterMaxPhaseBits = 6;         // intervals: a bucket in registers (at most 1,700 candidates of three
+                                                    // keys) takes fourteen tables of candidates at most
 constexpr uint64_t kFilterManyMinKeys = 1 << 16;    // fewest keys of a check of more than 16 intervals on this path
 constexpr uint64_t kFilterOnePassKeys = 64 * 1024;  // ... and at most, where one partition pass does
+constexpr uint32_t kFilterOnePassTables = 2;        // ... with at most so many tables of candidates
+constexpr uint32_t kFilterHalfThreadBits = 15;      // thread bits of a 16-bit entry of such a table
 
 struct BucketPlan {
   bool on = false;
@@ -378,8 +393,9 @@ struct BucketPlan {
 // (at most 2^kBucketMaxBits buckets of about kBucketTarget keys), its digit
 // widths, and its workspace section laid out from byte offset `off`
 // filter_ok: the model admits the table test (no warp or grid barriers, at most kFilterMaxLowBits key bits below the cell)
-bool plan_buckets(uint64_t n, uint64_t n_expect, uint32_t cb, uint32_t phase_bits, bool filter_ok, size_t off,
-                  BucketPlan* bp);
+// cells: at most as many cells hold keys; phase_bits, thread_bits: the key's fields
+bool plan_buckets(uint64_t n, uint64_t n_expect, uint32_t cb, uint64_t cells, uint32_t phase_bits, uint32_t thread_bits,
+                  bool filter_ok, size_t off, BucketPlan* bp);
 
 
 struct WorkspacePlan {

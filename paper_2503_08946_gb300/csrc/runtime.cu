@@ -227,24 +227,27 @@ static bool filter_allowed(bool sync_scopes, uint32_t cell_shift) {
   return !sync_scopes && cell_shift <= kFilterMaxLowBits;
 }
 
-// n key slots, of which about n_expect are kept (a hash-partitioned check keeps
-// its share): the bucket count is chosen for n_expect, the tile bounds for n
-// Bucket bits of the table test, or ~0 where it does not apply.
-static uint32_t filter_bucket_bits(uint64_t n_expect, uint32_t cb) {
+// Bucket bits of the cell test, or ~0 where it does not apply.
+static uint32_t filter_bucket_bits(uint64_t n_expect, uint32_t cb, uint64_t cells, uint32_t phase_bits,
+                                   uint32_t thread_bits) {
   uint32_t D = 0;
   while (D < cb && D < kBucketMaxBits && (n_expect >> D) > kFilterTarget) ++D;
   if (D == kBucketMaxBits && (n_expect >> D) > kFilterTarget) return ~0u;
   const uint32_t need = cb > kFilterMaxSlotBits ? cb - kFilterMaxSlotBits : 0u;   // for a slot per cell
-  // one partition pass where its buckets stay small enough to be read again from L2
+  // one partition pass where its buckets are read again a few times at most (rc_internal.h)
   const uint32_t one = kBucketMaxDigitBits;
-  if (D > one && need <= one && (n_expect >> one) <= kFilterOnePassKeys) return one;
+  const uint64_t table = 1ull << (kFilterMaxSlotBits + (thread_bits <= kFilterHalfThreadBits ? 1u : 0u));
+  const uint64_t entries = (cells >> one) << phase_bits;
+  if (D > one && need <= one && (n_expect >> one) <= kFilterOnePassKeys && entries <= kFilterOnePassTables * table) return one;
   if (need <= D) return D;
   if (need <= kBucketMaxBits && (n_expect >> need) >= kFilterMinKeys) return need;
   return cb - D <= kFilterMaxTagBits ? D : ~0u;   // a sparse cell space: hashed tables
 }
 
-bool plan_buckets(uint64_t n, uint64_t n_expect, uint32_t cb, uint32_t phase_bits, bool filter_ok, size_t off,
-                  BucketPlan* bp) {
+// n key slots, of which about n_expect are kept (a hash-partitioned check keeps
+// its share): the bucket count is chosen for n_expect, the tile bounds for n
+bool plan_buckets(uint64_t n, uint64_t n_expect, uint32_t cb, uint64_t cells, uint32_t phase_bits, uint32_t thread_bits,
+                  bool filter_ok, size_t off, BucketPlan* bp) {
   *bp = BucketPlan();
   if (n == 0 || n >= (1ull << 32) || cb == 0 || cb > 62) return false;
   // more than 16 intervals: the cell test only (the scan keeps masks of 16), where
@@ -252,7 +255,7 @@ bool plan_buckets(uint64_t n, uint64_t n_expect, uint32_t cb, uint32_t phase_bit
   const bool many = phase_bits > kScanTablePhaseBits;
   if (many && (phase_bits > kFilterMaxPhaseBits || n < kFilterManyMinKeys)) return false;
   if (n_expect == 0 || n_expect > n) n_expect = n;
-  uint32_t D = filter_ok ? filter_bucket_bits(n_expect, cb) : ~0u;
+  uint32_t D = filter_ok ? filter_bucket_bits(n_expect, cb, cells, phase_bits, thread_bits) : ~0u;
   bp->filter = D != ~0u;
   if (!bp->filter && many) return false;
   if (!bp->filter) {
@@ -319,8 +322,8 @@ void plan_workspace_keys(const Model& m, const rc_check_opts* opts, uint64_t n, 
   const uint32_t part_bits = part ? bit_length(opts->part_count - 1) : 0u;
   const uint64_t n_expect = part ? n / opts->part_count + n / (16ull * opts->part_count) + 1 : n;
   if (allow_bucket && bucket_path_allowed(opts) && cell_bits > part_bits &&
-      plan_buckets(n, n_expect, cell_bits - part_bits, m.host.phase_bits,
-                   filter_allowed(m.sync_scopes, m.host.cell_shift), off, &p->bucket)) {
+      plan_buckets(n, n_expect, cell_bits - part_bits, m.total_cells / (part ? opts->part_count : 1u), m.host.phase_bits,
+                   m.host.thread_bits, filter_allowed(m.sync_scopes, m.host.cell_shift), off, &p->bucket)) {
     // the bucket path: its own section instead of the radix-sort sections
     p->zero_lo = p->bucket.zero_lo;
     p->zero_hi = p->bucket.zero_hi;
@@ -1037,7 +1040,8 @@ rc_status enqueue_chunked(rc_model* model, const rc_check_opts* opts, uint8_t* w
       // sort's scratch (a chunk's keys hold no padding)
       const uint32_t ccb = hi - m.host.cell_shift;
       if (bucket_ok && c.n > 0 && m.host.cell_shift <= hi &&
-          rc::plan_buckets(c.n, c.n, ccb, m.host.phase_bits, true, pc.zero_lo, &p.bucket) && p.bucket.filter &&
+          rc::plan_buckets(c.n, c.n, ccb, c.span, m.host.phase_bits, m.host.thread_bits, true, pc.zero_lo, &p.bucket) &&
+          p.bucket.filter &&
           p.bucket.end <= pc.long_off) {
         s = cuda_status(rc::launch_init_check(res, k > wv.k0 ? 1u : 0u, nullptr, region + p.bucket.zero_lo,
                                               p.bucket.zero_hi - p.bucket.zero_lo, nullptr, st));
@@ -1255,7 +1259,8 @@ rc_status plan_batch(rc_model* const* models, size_t n, const rc_check_opts* opt
     p.keys_off[1] = o;
     o = align256(o + k.n_keys * 8);
     if (rc::bucket_path_allowed(opts) &&
-        rc::plan_buckets(k.n_keys, k.n_keys, k.cell_bits, k.pb, rc::filter_allowed(k.sy, ps + k.pb), o, &p.bucket)) {
+        rc::plan_buckets(k.n_keys, k.n_keys, k.cell_bits, k.total_cells, k.pb, k.tb,
+                         rc::filter_allowed(k.sy, ps + k.pb), o, &p.bucket)) {
       p.zero_lo = p.bucket.zero_lo;
       p.zero_hi = p.bucket.zero_hi;
       o = p.bucket.end;
