@@ -226,8 +226,10 @@ __device__ __forceinline__ void filter_bucket(const FilterArgs& a, const uint64_
       *reinterpret_cast<uint4*>(s_tag + i) = make_uint4(kNoTag, kNoTag, kNoTag, kNoTag);
   for (unsigned i = tid; i < (AT ? 10 : 4) * mw + 1; i += kFltThreads) s_two[i] = 0;
   __syncthreads();
+  bool any = false;
   if constexpr (HT) {
-    // 0. a slot for every written cell, then every key's slot
+    // 1. a slot for every written cell and its representative (in one reading of a
+    // larger bucket), then, when all have one, every key's slot
     bool full = false;
     each([&](unsigned k, unsigned tag) {
       if ((k & kmask) == 0u) return;
@@ -237,27 +239,33 @@ __device__ __forceinline__ void filter_bucket(const FilterArgs& a, const uint64_
         if (t == kNoTag) t = atomicCAS(&s_tag[i], kNoTag, tag);
         if (t == kNoTag || t == tag) break;
       }
-      full = full || n == kProbes;
-    });
-    if (__syncthreads_or(full)) return false;
-    resolve = true;
-    if constexpr (REGS) {
-#pragma unroll
-      for (int q = 0; q < kFltKPT; ++q) {
-        if (q >= nq) break;
-        rs[q] = find(rs[q]);
+      if (n == kProbes) {
+        full = true;
+        return;
       }
+      s_tab[i] = k;
+      any = true;
+    });
+    if constexpr (!REGS)
+      if (__syncthreads_or(full)) return false;
+    resolve = true;
+  } else {
+    // 1. the representative of every written cell (its low word is not 0)
+    each([&](unsigned k, unsigned s) {
+      if (k & kmask) {
+        s_tab[s] = k;
+        any = true;
+      }
+    });
+  }
+  if (!__syncthreads_or(any)) return true;   // no write: nothing can race
+  if constexpr (HT && REGS) {
+#pragma unroll
+    for (int q = 0; q < kFltKPT; ++q) {
+      if (q >= nq) break;
+      rs[q] = find(rs[q]);
     }
   }
-  // 1. the representative of every written cell (its low word is not 0)
-  bool any = false;
-  each([&](unsigned k, unsigned s) {
-    if (k & kmask) {
-      s_tab[s] = k;
-      any = true;
-    }
-  });
-  if (!__syncthreads_or(any)) return true;   // no write: nothing can race
   // 2. every key against its cell's representative
   any = false;
   each([&](unsigned k, unsigned s) {
