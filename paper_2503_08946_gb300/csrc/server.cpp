@@ -116,12 +116,21 @@ struct rc_server {
   rc_status fatal = RC_OK;
   std::thread th;
 
-  void finish(Slot& sl) {
+  // The scheduler thread alone touches the slots and the pool; mu guards the queues
+  // and counters that other threads see.  Everything that takes longer than moving
+  // requests (planning and enqueueing a batch, reading one back) runs without it, so
+  // that a submitting thread does not wait for them.
+  using Lock = std::unique_lock<std::mutex>;
+
+  // Called with mu held, which is released while the results are read.
+  void finish(Slot& sl, Lock& lk) {
+    lk.unlock();
     std::vector<rc_result> out(sl.reqs.size());
     const rc_status st = rc_report(sl.ticket, out.data(), 1);
     const double t = now_s();
+    std::vector<rc_server_done> ds(sl.reqs.size());
     for (size_t i = 0; i < sl.reqs.size(); ++i) {
-      rc_server_done d;
+      rc_server_done& d = ds[i];
       std::memset(&d, 0, sizeof(d));
       d.request = sl.reqs[i].id;
       d.result = out[i];
@@ -130,13 +139,15 @@ struct rc_server {
       d.start_s = sl.start_s;
       d.done_s = t;
       d.batch_size = (uint32_t)sl.reqs.size();
-      done.push_back(d);
     }
     pool.release(sl.ws_off, sl.ws_bytes);
-    in_flight -= sl.reqs.size();
-    sl.reqs.clear();
     sl.ticket = nullptr;
     sl.busy = false;
+    lk.lock();
+    done.insert(done.end(), ds.begin(), ds.end());
+    in_flight -= sl.reqs.size();
+    sl.reqs.clear();
+    cv_done.notify_all();
   }
 
   void fail_now(const Request& r, rc_status st) {
@@ -159,17 +170,20 @@ struct rc_server {
     return b;
   }
 
-  // Admit waiting requests into free slots.  Called with mu held.
-  void admit() {
+  // Admit waiting requests into free slots.  Called with mu held, which is released
+  // while a batch is planned and enqueued (requests are only added to the queue
+  // meanwhile: its front is the scheduler's to take).
+  void admit(Lock& lk) {
     for (Slot& sl : slots) {
       if (sl.busy || pending.empty()) continue;
-      // the longest prefix of the queue (at most max_batch) whose batch fits the
-      // largest free block, by binary search over the prefix length
-      const size_t room = pool.largest();
       const size_t cap = std::min<size_t>(pending.size(), opts.max_batch ? opts.max_batch : 1024);
       std::vector<rc_model*> all;
       all.reserve(cap);
       for (size_t i = 0; i < cap; ++i) all.push_back(pending[i].model);
+      lk.unlock();
+      // the longest prefix of the queue (at most max_batch) whose batch fits the
+      // largest free block, by binary search over the prefix length
+      const size_t room = pool.largest();
       size_t lo = 0, hi = cap, need = 0;
       while (lo < hi) {
         const size_t mid = (lo + hi + 1) / 2;
@@ -185,8 +199,10 @@ struct rc_server {
       std::vector<rc_model*> ms(all.begin(), all.begin() + (long)lo);
       if (ms.empty()) {
         // the oldest request does not fit now; if it cannot fit at all, fail it
-        std::vector<rc_model*> one{pending.front().model};
-        if (need_for(one) > opts.memory_bytes) {
+        std::vector<rc_model*> one{all.front()};
+        const bool never = need_for(one) > opts.memory_bytes;
+        lk.lock();
+        if (never) {
           fail_now(pending.front(), RC_E_NOMEM);
           pending.pop_front();
           cv_done.notify_all();
@@ -194,17 +210,23 @@ struct rc_server {
         return;
       }
       const size_t off = pool.alloc(need);
+      lk.lock();
       if (off == SIZE_MAX) return;
       sl.reqs.assign(pending.begin(), pending.begin() + (long)ms.size());
       pending.erase(pending.begin(), pending.begin() + (long)ms.size());
+      in_flight += sl.reqs.size();
+      lk.unlock();
       rc_check_opts o{};
       o.path = RC_PATH_SORT;
       o.digit_bits = opts.digit_bits;
       rc_ticket t = nullptr;
       const rc_status st = rc_check_batch(ms.data(), ms.size(), &o, pool_base + off, need, sl.stream, &t);
+      if (st != RC_OK) pool.release(off, need);
+      const double now = now_s();
+      lk.lock();
       if (st != RC_OK) {
-        pool.release(off, need);
         for (const Request& r : sl.reqs) fail_now(r, st);
+        in_flight -= sl.reqs.size();
         sl.reqs.clear();
         cv_done.notify_all();
         continue;
@@ -212,31 +234,26 @@ struct rc_server {
       sl.ticket = t;
       sl.ws_off = off;
       sl.ws_bytes = need;
-      sl.start_s = now_s();
+      sl.start_s = now;
       sl.busy = true;
-      in_flight += sl.reqs.size();
     }
   }
 
   void loop() {
     cudaSetDevice(device);
-    std::unique_lock<std::mutex> lk(mu);
+    Lock lk(mu);
     while (true) {
-      bool progressed = false;
       for (Slot& sl : slots) {
         if (!sl.busy) continue;
         const cudaError_t q = cudaStreamQuery(sl.stream);
         if (q == cudaSuccess) {
-          finish(sl);
-          progressed = true;
+          finish(sl, lk);
         } else if (q != cudaErrorNotReady) {
           fatal = RC_E_CUDA;
-          finish(sl);
-          progressed = true;
+          finish(sl, lk);
         }
       }
-      if (progressed) cv_done.notify_all();
-      admit();
+      admit(lk);
       bool any_busy = false;
       for (Slot& sl : slots) any_busy |= sl.busy;
       if (stop && !any_busy && pending.empty()) break;
