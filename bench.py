@@ -59,7 +59,7 @@ def load_peaks():
 
 
 KERNEL_SOURCES = {"onesweep": "sort.cu", "partition": "sort.cu", "partition_a": "bucket.cu",
-                  "partition_b": "bucket.cu", "cell_test": "filter.cu", "histogram_b": "bucket.cu",
+                  "partition_b": "bucket.cu", "cell_test": "filter.cu", "histogram_b": "bucket.cu", "local_sort": "bucket.cu",
                   "scan": "scan.cu", "expand": "jit.cpp", "histogram": "bucket.cu"}
 
 
@@ -296,9 +296,12 @@ def run_native(args):
     # per kernel: (algorithmic bytes per launch, mean launch ms).  Every pass
     # (partition, radix pass) reads and writes each key once (16 B per key);
     # expansion writes 8 B, histograms, the cell test and the scan read 8 B.
+    # (The model has no warp or grid barriers: the bucket path ends in the cell test
+    # if the fields below the cell fit its 32-bit words, else in local sort and scan.)
+    cell_test = lay["cell_shift"] <= 32
     if bucketed:
-        names = {3: ["partition_a", "partition_b", "cell_test"], 2: ["partition_a", "cell_test"],
-                 1: ["cell_test"]}[n_pass]
+        last = "cell_test" if cell_test else "local_sort"
+        names = {3: ["partition_a", "partition_b", last], 2: ["partition_a", last], 1: [last]}[n_pass]
         kern = {nm: ((8.0 if nm == "cell_test" else 16.0) * n_keys, st_mean["sort_pass_ms"][i])
                 for i, nm in enumerate(names)}
         if n_pass == 3:
@@ -311,7 +314,7 @@ def run_native(args):
     hist_fused = bool(stages[0].get("histogram_fused"))
     if not hist_fused:   # (else the expansion counted it: no pass over the keys)
         kern["histogram"] = (8.0 * n_keys, st_mean["histogram_ms"])
-    if not bucketed:   # (the cell test has no scan)
+    if not bucketed or not cell_test:   # (the cell test has no scan)
         kern["scan"] = (8.0 * n_keys, st_mean["scan_ms"])
     launches = {"onesweep": max(1, n_pass - 1)} if not bucketed else {}
     dominant = max(kern, key=lambda k: kern[k][1] * launches.get(k, 1))
@@ -325,8 +328,9 @@ def run_native(args):
     per_kernel = {k: {"ms": v[1], "alg_bytes_per_key": v[0] / n_keys,
                       "frac": v[0] / (v[1] / 1e3) / 1e9 / peak if v[1] > 0 else None} for k, v in kern.items()}
     # the whole check: expansion 8, histograms 8 each (none for a histogram the
-    # expansion counts), passes 16 each, cell test or scan 8 bytes per key
-    pk = 8 + (0 if hist_fused else 8) + 8 + (16 * (n_pass - 1) + (8 if n_pass == 3 else 0) if bucketed else 16 * n_pass)
+    # expansion counts), passes 16 each, cell test or scan 8 bytes per key, local sort 16
+    pk = 8 + (0 if hist_fused else 8) + 8 + (16 * (n_pass - 1) + (8 if n_pass == 3 else 0) + (0 if cell_test else 16)
+                                             if bucketed else 16 * n_pass)
     pipeline_bytes = pk * n_keys
     pipeline = {"alg_bytes_per_key": pk,
                 "gbs": pipeline_bytes / (st_mean["check_ms"] / 1e3) / 1e9,

@@ -343,8 +343,10 @@ enum { RC_OPT_STAGE_TIMES = 1, RC_OPT_GRAPH = 2, RC_OPT_CHUNKED = 4, RC_OPT_LSD 
  * keys carry at most 16 barrier intervals groups its keys by cell with the
  * bucket path: two look-back-free partition passes on the top bits of a
  * bijective hash of the cell, then, for models without warp or grid barriers
- * whose cells have a table slot each in their bucket, the cell test in shared
- * memory (also for up to 64 intervals when there are at least 2^16 keys), else a
+ * whose interval, block, thread and kind take at most 32 key bits, the cell test
+ * in shared memory (a table slot per cell of a bucket, or hashed tables where the
+ * cell space is sparse; also for up to 64 intervals when there are at least 2^16
+ * keys), else a
  * counting sort of every bucket in shared memory on the hash's remaining bits,
  * which leaves every cell's keys together (cells in hash order), and the cell
  * scan; the result is identical to the radix-sorted check's.

@@ -16,9 +16,10 @@
 //   sort    average kBucketTarget) is counting-sorted by the remaining bits of
 //           h in shared memory and written back, so that the keys of every
 //           cell are contiguous (the cells are in h order, not in cell order).
-// For models without atomics and scopes whose cells fit a table per bucket, the
-// local sort and the scan are replaced by the cell test of filter.cu.
-// Otherwise the ordered cell scan (scan.cu) then folds the cells; it needs each cell's
+// For models without warp or grid barriers whose fields below the cell fit 32 bits,
+// the cell test of filter.cu decides the buckets instead of the local sort and the
+// scan; one pass of 10 bits with larger buckets then does for many checks (pass A
+// alone).  Otherwise the ordered cell scan (scan.cu) folds the cells; it needs each cell's
 // keys together, in any order, and with `by_cell` keeps the smallest racy cell
 // by value (DevResult.hash_cell); bucket_finish points the witness kernels at
 // its bucket, whose keys they filter by cell.

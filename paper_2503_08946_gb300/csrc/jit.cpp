@@ -8,19 +8,22 @@
 // divisors as literals, so the compiler folds constants, hoists the
 // thread-constant expressions out of the loops and turns floor division and
 // modulo by constants into multiply-shift sequences (or masks and shifts for
-// powers of two).  The generated kernel writes exactly the keys of the
-// interpreted one (same slots, same padding, same out-of-bounds report).
+// powers of two).  With all points (rc_expand_keys) the generated kernel writes
+// exactly the keys of the interpreted one (same slots, same padding, same
+// out-of-bounds report).
 //
 // NVRTC and the CUDA driver entry points are resolved at run time (dlopen and
 // cudaGetDriverEntryPointByVersion), so the library loads on machines without
 // them; rc_model_create then keeps the interpreted expansion.  Compiled
 // kernels are cached per device by their source text.
 //
-// A check expands each statement's distinct points only (find_distinct_points):
-// the random affine model of 4096 x 256 threads makes 40 to 50 % of its keys
-// that way, and every later stage moves that much less.  Measured on it (578 M
-// keys of all points): the expansion 0.89 -> 0.71 ms (it now evaluates a point
-// from its number instead of stepping a loop), the check 7.2 -> 4.3 ms.
+// A check expands each statement's distinct points only (find_distinct_points), in
+// slots of their own (Model.check_slots instead of key_slots), and writes padding for
+// an access that repeats its instance in the innermost loop.  Random affine models of
+// 4096 x 256 threads keep 29 to 52 % of their keys, and every later stage moves that
+// much less.  Measured on one of them (303 of 578 M keys): the expansion 0.89 -> 0.71
+// ms (it evaluates a point from its number instead of stepping a loop), the check
+// 7.2 -> 4.3 ms.
 #include <cuda.h>
 #include <cuda_runtime_api.h>
 #include <dlfcn.h>
